@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "fbsde_kernels.cuh"
+#include "fbsde_cg.cuh"
 #include "fbsde_matvec.cuh"
 
 namespace fbsde {
@@ -17,26 +18,147 @@ namespace {
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Team geometry: a row of nch 16-byte chunks is covered by tw warps holding vpt
-// chunks per thread; narrow rows use one warp per row and 8 rows per CTA.  Rows of more
-// than 4096 chunks (FP64 rows beyond 8192 values) take 16 chunks per thread, so that their
-// team stays within 16 warps.
-bool choose_team(int nch, int &tw, int &vpt, int &teams)
+// Team geometry: a row of nch 16-byte chunks is covered by tw warps holding vpt chunks per
+// thread.  Rows that stay in shared memory take at most 4 chunks per thread up to 1792 chunks
+// (14 warps, and registers for two rows held at a time): many short row steps in flight.
+// Rows that stream take up to 8 (fewer warps, barriers and butterflies per byte), and more
+// than 4096 chunks (FP64 rows beyond 8192 values) 16, so that a team stays within 16 warps.
+bool choose_team(int nch, bool resident, int &tw, int &vpt)
 {
-    constexpr int vmax = 8;
-    if (nch <= 32 * vmax) {
-        tw = 1;
-        vpt = 1;
-        while (32 * vpt < nch) vpt *= 2;
-    } else if (nch <= 16 * 32 * vmax) {
-        vpt = vmax;
-        tw = (nch + 32 * vmax - 1) / (32 * vmax);
-    } else {
-        vpt = 2 * vmax;
-        tw = (nch + 32 * 2 * vmax - 1) / (32 * 2 * vmax);
+    vpt = 1;
+    while (vpt < 4 && 32 * vpt < nch) vpt *= 2;
+    if (nch > (resident ? 14 * 32 * 4 : 32 * 4)) vpt = nch <= 16 * 32 * 8 ? 8 : 16;
+    tw = (nch + 32 * vpt - 1) / (32 * vpt);
+    return 32 * tw <= 512;
+}
+
+// Ring of a product launch of G chunks per query: S stages of R rows, about 32 KB a stage and
+// 200 KB of shared memory in all.  A CTA never needs a ring larger than its own rows: small
+// instances keep their ring, and so their shared memory, small (two stages of at most half
+// their rows), which lets the CTAs of concurrent instances share an SM.
+void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, size_t real_sz,
+                  int &rows, int &stages, size_t &smem)
+{
+    const size_t stage_target = 32 * 1024, ring_target = 200 * 1024;
+    long long R = std::max<long long>(1, (long long)(stage_target / row_bytes));
+    R = std::max<long long>(teams, R / teams * teams);
+    long long S = std::min<long long>(8, std::max<long long>(2, ring_target / (R * row_bytes)));
+    const long long rows_cta = (P->M + G - 1) / G;
+    if (S * R > rows_cta) {
+        const long long half = ((rows_cta + 1) / 2 + teams - 1) / teams * teams;
+        R = std::min<long long>(R, std::max<long long>(teams, half));
+        S = std::max<long long>(2, std::min<long long>(S, (rows_cta + R - 1) / R));
     }
-    if (32 * tw > 512) return false;
-    teams = std::max(1, 256 / (32 * tw));
+    rows = (int)R;
+    stages = (int)S;
+    smem = (size_t)S * R * row_bytes + 2 * S * sizeof(uint64_t) + (size_t)teams * 2 * 32 * real_sz;
+}
+
+// Geometry of the CG (fbsde_cg.cuh): teams, chunks, tiles and the loop's shared memory; all
+// from the shape alone, so the order of every sum is the same in both forms and on any
+// device.
+//   - Chunks: without a given ctas, as many waves of 152 chunks (one per SM) over the
+//     queries as fill the SMs best, no chunk below one row per team (four rows for one
+//     team: a chunk's partial vector is written and read like a row).
+//   - A chunk that fits the loop's shared memory stays there for the whole loop; then up
+//     to 14 warps share its rows, which hides the latency of
+//     a row's dot product.  Rows that stream through the ring instead get as many teams as
+//     leave the ring four stages (the teams' sums need one row each).
+//   - Tiles: the narrowest of 4, 8, .. 128 coordinates that gives at most one tile per SM:
+//     the partial vectors of a tile are added by one CTA, so more tiles shorten phase B.
+constexpr size_t kCgSmem = 225 * 1024;   // dynamic shared memory of the loop
+constexpr long long kCgSms = 152;
+
+bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
+{
+    const size_t row = (size_t)L.ld * L.real_sz;
+    const int nch = (int)(row / 16);
+    if (!choose_team(nch, true, L.team_warps, L.vpt)) return false;
+    // consumer warps of the loop's block beside the producer; with the rows resident a warp
+    // more is left for the scalars
+    const int warps = L.vpt == 8 ? 10 : 14;
+    // (two stages of one row per team also fit the product's own ring)
+    const int tmax = (int)std::max<long long>(
+        1, std::min<long long>(warps / L.team_warps, 96 * 1024 / (long long)row));
+    const size_t tile_sm = L.precision == FBSDE_FP32 ? sizeof(dev::CgTileSm<float>)
+                                                     : sizeof(dev::CgTileSm<double>);
+    auto fixed = [&](int teams, long long ring_rows, int stages) {   // all but the ring
+        L.cg_op = teams > 1 ? 1 : 0;
+        L.cg_both = (int)align_up(std::max(tile_sm, teams > 1 ? teams * row : 0), 16);
+        return (size_t)L.cg_op * row + L.cg_both + Q * sizeof(dev::CgScal) + 16 * (size_t)stages +
+               ((size_t)teams * 64 + ring_rows) * L.real_sz + 128;
+    };
+    auto chunks = [&](int teams, bool one_wave) {
+        const long long gmax =
+            std::max<long long>(1, P->ctas > 0 ? P->M / kMinRowsPerCta : P->M / (teams > 1 ? teams : 4));
+        if (P->ctas > 0) return (int)std::min<long long>(gmax, (P->ctas + Q - 1) / Q);
+        double best = -1.0;
+        int G = 1;
+        for (int W = 1; W <= (one_wave ? 1 : 8); ++W) {
+            const long long g = std::min(gmax, std::max<long long>(1, kCgSms * W / Q));
+            const double waves = (double)(g * Q) / kCgSms, eff = waves / std::ceil(waves);
+            if (eff > best + 0.015) {
+                best = eff;
+                G = (int)g;
+            }
+            if (g == gmax) break;
+        }
+        return G;
+    };
+    const int gcap = kPartVecs * std::max(L.G, L.Gs);   // the partial vectors' buffer
+    int wmax = warps;
+    L.cg_res = 0;
+    L.teams = tmax;
+    L.Gc = std::min(gcap, chunks(tmax, true));
+    long long rows = (P->M + L.Gc - 1) / L.Gc;
+    if ((long long)Q * L.Gc <= kCgSms && L.team_warps <= warps && L.vpt <= 8 &&
+        rows * row + fixed(tmax, rows, 2) <= kCgSmem) {
+        L.cg_res = 1;
+        L.cg_stages = rows > tmax ? 2 : 1;
+        L.cg_rows = (int)((rows + L.cg_stages - 1) / L.cg_stages + tmax - 1) / tmax * tmax;
+        L.cg_ring = (int)rows;
+        L.cg_smem = rows * row + fixed(tmax, rows, L.cg_stages);
+    } else {
+        if (!choose_team(nch, false, L.team_warps, L.vpt)) return false;
+        wmax = L.vpt >= 8 ? 10 : 15;
+        L.teams = (int)std::max<long long>(
+            1, std::min<long long>(wmax / L.team_warps, 32 * 1024 / (long long)row));
+        L.Gc = std::min(gcap, chunks(L.teams, false));
+        rows = (P->M + L.Gc - 1) / L.Gc;
+        const long long R = std::max<long long>(1, 32 * 1024 / (long long)row / L.teams) * L.teams;
+        const size_t rest = fixed(L.teams, 0, 8);
+        const long long S = rest < kCgSmem ? std::min<long long>(8, (kCgSmem - rest) / (R * row)) : 0;
+        L.cg_rows = (int)R;
+        L.cg_stages = (int)S;
+        L.cg_ring = (int)(R * S);
+        L.cg_smem = R * S * row + fixed(L.teams, 0, (int)S);
+    }
+    L.cg_ok = Q <= dev::kCgQueries && L.team_warps <= wmax && L.vpt <= 8 && L.cg_stages >= (L.cg_res ? 1 : 2) &&
+              L.cg_smem <= kCgSmem;
+    // Several queries whose rows stream have a pass per barrier as long as their rows: from
+    // about 0.6 GB on (d = 10^4, 16 queries: 1445 us a pass in the loop, 1400 us in two
+    // launches; d = 1000, 64 queries, 1.05 GB: 197 and 189 us; 16 queries, 0.26 GB: 57 and
+    // 75 us) its launches cost less than the loop's fixed split of the chunks over the SMs.
+    if (!L.cg_res && Q > 1 && (double)Q * P->M * row > 6e8) L.cg_ok = 0;
+    // FP32 shapes of the three-launch pass (fbsde_cg3.cuh), in its own geometry
+    L.cg3 = L.precision == FBSDE_FP32 && (L.sde || (!L.cg_ok && L.teams == 1));
+    if (L.cg3) {
+        L.c3_vpt = 1;
+        while (L.c3_vpt < 8 && 32 * L.c3_vpt < nch) L.c3_vpt *= 2;
+        L.c3_tw = (nch + 32 * L.c3_vpt - 1) / (32 * L.c3_vpt);
+        L.c3_teams = std::max(1, 256 / (32 * L.c3_tw));
+        product_ring(P, row, L.G, L.c3_teams, 4, L.c3_rows, L.c3_stages, L.c3_smem);
+        if (L.c3_tw > 16 || L.c3_smem > 227 * 1024) return false;
+    }
+    L.mv_mode = L.team_warps > 10 ? dev::kMvWide : (L.teams > 1 ? dev::kMvHold : dev::kMvPair);
+    L.threads = L.teams * 32 * L.team_warps;
+    L.cg_lpr = 32;
+    for (int lpr : {1, 2, 4, 8, 16})
+        if ((long long)Q * ((L.ld + 4 * lpr - 1) / (4 * lpr)) <= kCgSms) {
+            L.cg_lpr = lpr;
+            break;
+        }
+    L.cg_nblk = (L.ld + 4 * L.cg_lpr - 1) / (4 * L.cg_lpr);
     return true;
 }
 
@@ -109,8 +231,6 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     L.ld = (P->d + 3) / 4 * 4;
     L.real_sz = P->precision == FBSDE_FP32 ? sizeof(float) : sizeof(double);
     const int nch = (int)(L.ld * L.real_sz / 16);
-    if (!choose_team(nch, L.team_warps, L.vpt, L.teams)) return FBSDE_ERR_ARG;
-    L.threads = L.teams * 32 * L.team_warps;
     const long long gmax = std::max<long long>(1, P->M / kMinRowsPerCta);
     const int target = P->ctas > 0 ? P->ctas : kTargetCtas;
     L.G = (int)std::min<long long>(gmax, std::max(1, (target + Q - 1) / Q));
@@ -121,29 +241,6 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
                                             (long long)kRowBlocks);
     // per-particle kernel: 256 particles per block
     L.GP = (int)((P->M + 255) / 256);
-    // matrix-free product: ring of mv_stages stages of mv_rows rows (~32 KB per stage,
-    // ~200 KB of shared memory in total)
-    {
-        const size_t row_bytes = (size_t)L.ld * L.real_sz;
-        const size_t stage_target = 32 * 1024, ring_target = 200 * 1024;
-        long long R = std::max<long long>(1, (long long)(stage_target / row_bytes));
-        R = std::max<long long>(L.teams, R / L.teams * L.teams);
-        long long S = std::min<long long>(8, std::max<long long>(2, ring_target / (R * row_bytes)));
-        // a CTA never needs a ring larger than its own rows: small instances keep their
-        // ring, and so their shared memory, small (two stages of at most half their rows),
-        // which lets the CTAs of concurrent instances share an SM
-        const long long rows_cta = (P->M + L.G - 1) / L.G;
-        if (S * R > rows_cta) {
-            const long long half = ((rows_cta + 1) / 2 + L.teams - 1) / L.teams * L.teams;
-            R = std::min<long long>(R, std::max<long long>(L.teams, half));
-            S = std::max<long long>(2, std::min<long long>(S, (rows_cta + R - 1) / R));
-        }
-        L.mv_rows = (int)R;
-        L.mv_stages = (int)S;
-        L.mv_smem = (size_t)L.mv_stages * R * row_bytes + 2 * L.mv_stages * sizeof(uint64_t) +
-                    (size_t)L.teams * 2 * 32 * L.real_sz;
-        if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
-    }
     // fused per-level step (FP32 rows up to kStepMaxLd floats): R rows per stage, the
     // largest of {1, 3, 5, 15, 30} with R ld <= kStepElems (at most 30: one service-warp lane
     // per row), T = 480 / R threads per row in the row pass (whole warps, or half-warps at
@@ -190,6 +287,10 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
             if (eff >= 0.99) break;
         }
     }
+    if (!cg_geometry(P, Q, L)) return FBSDE_ERR_ARG;
+    product_ring(P, (size_t)L.ld * L.real_sz, L.Gc, L.teams, L.real_sz, L.mv_rows, L.mv_stages,
+                 L.mv_smem);
+    if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
     L.GS = std::max(L.GP, L.fused ? L.Gs : 0);
     // partial reduction: tiles of kRedTile elements, red_groups warps per tile, each adding
     // about four of the G partials
@@ -307,7 +408,19 @@ Params make_params(const fbsde_problem *P, const Layout &L, void *ws, uint64_t s
     p.vecR = base + L.off_vecR;
     p.st = reinterpret_cast<SolveState *>(base + L.off_state);
     p.bpart = reinterpret_cast<double *>(base + L.off_bpart);
-    p.nblk = L.nblk;
+    p.nblk3 = L.nblk;
+    p.bar = reinterpret_cast<unsigned int *>(base + L.off_bpart);
+    p.dpart = reinterpret_cast<double *>(base + L.off_segp);
+    p.part_vecs = kPartVecs;
+    p.nblk = L.cg_nblk;
+    p.cg_teams = L.teams;
+    p.cg_lpr = L.cg_lpr;
+    p.cg_rows = L.cg_rows;
+    p.cg_stages = L.cg_stages;
+    p.cg_ring = L.cg_ring;
+    p.cg_res = L.cg_res;
+    p.cg_op = L.cg_op;
+    p.cg_both = L.cg_both;
     p.u0 = u0;
     p.grad = grad;
     if (tr) {
@@ -367,12 +480,24 @@ bool profiling_products()
 // into a CUDA graph being captured on that stream, with each CG loop as a conditional
 // while node whose body is captured on a second stream.  graph_tail (eager only): the
 // CG passes that the eager loop does not launch one by one run as a cached CUDA graph.
+// branches: parallel graph branches of the capture (the CG loop's cooperative launch fills
+// the GPU, so only a capture of one branch takes it).
 struct Rec {
     cudaStream_t s;
     bool capture;
     cudaStream_t body;
     bool graph_tail;
+    int branches = 1;
 };
+
+// The parameters as the CG's kernels see them: the product's chunks, one vector per partial.
+Params product_params(const Params &p, const Layout &L)
+{
+    Params q = p;
+    q.G = L.Gc;
+    q.part_vecs = 1;
+    return q;
+}
 
 #define FBSDE_TRY(fam, call)                                                                 \
     do {                                                                                     \
@@ -383,9 +508,9 @@ struct Rec {
 constexpr int kCgUnroll = 2;   // CG passes per iteration of the conditional while node
 
 // The CG loop captured into the graph being built on stream s: a reset kernel that sets
-// the loop condition, then a conditional while node whose body (product, reduction, CG
-// update) is captured on the stream `body`; k_cg_update keeps the condition at 1 while
-// some query iterates and fewer than cg_max_iter passes ran.
+// the loop condition, then a conditional while node whose body (product, CG tiles) is
+// captured on the stream `body`; k_cg_tile keeps the condition at 1 while some query
+// iterates and fewer than cg_max_iter passes ran.
 template <typename Real>
 cudaError_t cg_capture(const Params &p, const Layout &L, cudaStream_t s, cudaStream_t b)
 {
@@ -422,9 +547,12 @@ cudaError_t cg_capture(const Params &p, const Layout &L, cudaStream_t s, cudaStr
     // once (the kernels test the query's done flag), and every pass updates the condition
     cudaError_t eb = cudaSuccess;
     for (int u = 0; u < kCgUnroll && eb == cudaSuccess; ++u) {
+        if (L.cg3) {
+            for (int k = 0; k < 3 && eb == cudaSuccess; ++k) eb = LR::cg3(p, L, k, h, 1, b);
+            continue;
+        }
         eb = LR::matvec(p, L, b);
-        if (eb == cudaSuccess) eb = LR::reduce(p, L, 1, 5, 1, b);
-        if (eb == cudaSuccess) eb = LR::cg_update(p, L, h, 1, b);
+        if (eb == cudaSuccess) eb = LR::cg_tile(p, L, h, 1, b);
     }
     cudaGraph_t ended = nullptr;
     e = cudaStreamEndCapture(b, &ended);
@@ -515,20 +643,24 @@ template <typename Real> cudaError_t cg_graph_launch(const Params &p, const Layo
     return cudaEventRecord(it->last, s);
 }
 
-// The CG iterations of one regression (all queries of the launch together).  Eager: the
-// passes are launched one by one (kernels of queries that have converged exit at once),
-// or, with graph_tail, handed to a cached CUDA graph whose conditional while loop runs
-// only the passes some query needs.  While the launch profiler times the product kernel,
-// the first kEagerPasses passes stay eager so their products can be bracketed by events.
-// A stream that is itself being captured gets the eager passes.
-template <typename Real> cudaError_t cg_loop(const Params &p, const Layout &L, const Rec &r)
+// The CG iterations of one regression (all queries of the launch together): one cooperative
+// launch of the whole loop wherever the shape has one and the work does not share the GPU
+// with other branches of a plan.  Otherwise a conditional while loop of the two phases:
+// captured into the plan's graph, or (graph_tail) a cached CUDA graph, or, on a stream that
+// is itself being captured and without graph_tail, every pass launched one by one (kernels
+// of queries that have converged exit at once).  While the launch profiler times the product
+// kernel, the first kEagerPasses passes are launched one by one so that their products can
+// be bracketed by events.  Every form gives the same bits.
+template <typename Real> cudaError_t cg_loop(const Params &p0, const Layout &L, const Rec &r)
 {
     using LR = Launch<Real>;
     cudaError_t e;
     const cudaStream_t s = r.s;
-    if (r.capture) return cg_capture<Real>(p, L, s, r.body);
-    bool tail = r.graph_tail;
-    if (tail) {
+    const Params p = product_params(p0, L);
+    const bool one = r.branches == 1 && !L.cg3 && LR::cg_loop_fits(L);
+    if (r.capture) return one ? LR::cg_loop(p, L, s) : cg_capture<Real>(p, L, s, r.body);
+    bool tail = r.graph_tail || one;
+    if (tail && !one) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if ((e = cudaStreamIsCapturing(s, &cs)) != cudaSuccess) return e;
         tail = cs == cudaStreamCaptureStatusNone;
@@ -536,11 +668,18 @@ template <typename Real> cudaError_t cg_loop(const Params &p, const Layout &L, c
     const int eager = !tail ? p.cg_max_iter
                             : (profiling_products() ? std::min(p.cg_max_iter, kEagerPasses) : 0);
     for (int it = 0; it < eager; ++it) {
+        if (L.cg3) {
+            FBSDE_TRY(FBSDE_K_MATVEC, LR::cg3(p, L, 0, 0, 0, s));
+            FBSDE_TRY(FBSDE_K_REDUCE, LR::cg3(p, L, 1, 0, 0, s));
+            FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg3(p, L, 2, 0, 0, s));
+            continue;
+        }
         FBSDE_TRY(FBSDE_K_MATVEC, LR::matvec(p, L, s));
-        FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 1, 5, 1, s));
-        FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_update(p, L, 0, 0, s));
+        FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_tile(p, L, 0, 0, s));
     }
-    if (eager < p.cg_max_iter) return cg_graph_launch<Real>(p, L, s);
+    if (eager >= p.cg_max_iter) return cudaSuccess;
+    if (!one) return cg_graph_launch<Real>(p, L, s);
+    FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_loop(p, L, s));
     return cudaSuccess;
 }
 
@@ -572,7 +711,7 @@ cudaError_t run(Params p, const Layout &L, const double *x0, const double *theta
     }
     if (p.tr_x_N || p.tr_y_N) FBSDE_TRY(FBSDE_K_TRACE, LR::trace_forward(p, L, s));
     if (!L.fused) FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-    FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, 0, s));
+    FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, s));
     p.newton_level = -1;
     FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 0, s));
     for (int k = p.N - 1; k >= 0; --k) {
@@ -584,12 +723,12 @@ cudaError_t run(Params p, const Layout &L, const double *x0, const double *theta
                 ps = p;
                 ps.G = L.Gs;
                 FBSDE_TRY(FBSDE_K_STEP, LR::step(ps, L, s));
-                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, 0, s));
+                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, s));
             } else {
                 FBSDE_TRY(FBSDE_K_UPDATE, LR::update(p, L, s));
                 FBSDE_TRY(FBSDE_K_PARTICLES, LR::particles(p, L, s));
                 FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, 0, s));
+                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, s));
             }
             p.newton_level = k;
             FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 1, s));
@@ -635,7 +774,7 @@ cudaError_t run_sde(Params p, const Layout &L, const double *x0, const double *t
     FBSDE_TRY(FBSDE_K_PARTICLES, LR::particles(p, L, s));
     if (p.tr_x_N || p.tr_y_N) FBSDE_TRY(FBSDE_K_TRACE, LR::trace_forward(p, L, s));
     FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-    FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, 0, s));
+    FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, s));
     FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 0, s));
     for (int k = N - 1; k >= 0; --k) {
         p.level = k;
@@ -656,7 +795,7 @@ cudaError_t run_sde(Params p, const Layout &L, const double *x0, const double *t
         FBSDE_TRY(FBSDE_K_PARTICLES, LR::sde_rho(p, L, s));
         FBSDE_TRY(FBSDE_K_PARTICLES, LR::particles(p, L, s));
         FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-        FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, 0, s));
+        FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, s));
         p.newton_level = k;
         FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 1, s));
     }
@@ -702,8 +841,9 @@ cudaError_t run_adjoint(Params p, const Layout &L, const double *x0, const doubl
         }
         if (k >= 1) {   // start from the previous level's solution: one product
             FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_warm(p, L, s));
-            FBSDE_TRY(FBSDE_K_MATVEC, LR::matvec(p, L, s));
-            FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 1, 5, 0, s));
+            const Params q = L.cg3 ? p : product_params(p, L);
+            FBSDE_TRY(FBSDE_K_MATVEC, L.cg3 ? LR::cg3(q, L, 0, 0, 0, s) : LR::matvec(q, L, s));
+            FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(q, L, 1, 5, s));
         }
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_setup(p, L, k >= 1 ? 1 : 0, s));
         if ((e = cg_loop<Real>(p, L, r)) != cudaSuccess) return e;
@@ -714,7 +854,7 @@ cudaError_t run_adjoint(Params p, const Layout &L, const double *x0, const doubl
         const bool terminal = k + 1 == p.N;
         const int mb = terminal ? mode_b : (p.kind == FBSDE_AC_MANUFACTURED ? 1 : 0);
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_colsum(p, L, mb, terminal ? mode_c : 0, s));
-        FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, 0, s));
+        FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, s));
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_finalize(p, L, s));
         if (!terminal) {  // rows Delta_{k+1} -> Delta_{k+2}: the bridge step of level k+1 inverted
             Params q = p;
@@ -1033,7 +1173,7 @@ int fbsde_plan_create(fbsde_plan **plan, int32_t n, const fbsde_instance *inst, 
     for (int b = 0; b < B && e == cudaSuccess; ++b)
         e = cudaStreamWaitEvent(pl->streams[2 + b], pl->events[0], 0);
     for (int b = 0; b < B && e == cudaSuccess; ++b) {
-        const Rec r{pl->streams[2 + b], true, body, false};
+        const Rec r{pl->streams[2 + b], true, body, false, B};
         for (int i : lists[b]) {
             const PlanInstance &pi = v[i];
             void *ws = static_cast<char *>(workspace) + pi.offset;

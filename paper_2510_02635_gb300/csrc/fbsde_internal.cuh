@@ -6,9 +6,11 @@
 //   w      [Q][M]          Real   kernel weight of particle j in the current regression
 //   coef   [Q][M][3]       Real   moment coefficients (w, w (Y - yref), w D.x_ws)
 //   segp   [Q][M][nseg][6] Real   per-row-segment partial sums of the row kernels
-//   part   [Q][G][3][ld]   Real   per-CTA partial d-vectors (moments or the CG product)
+//   part   [Q][G][3][ld]   Real   per-CTA partial d-vectors of the moments, or [Q][Gc][ld] of
+//                                 the CG product
 //   spart  [Q][GS][4]      double per-particle-block partial scalars
-//   vec64  [Q][9][ld]      double x (= alpha_x), r, p, S, b/rhs, q/G, x0, s, previous alpha_x
+//   vec64  [Q][9][ld]      double x (= alpha_x), r, p, S, b/rhs, G / shares of the CG, x0, s,
+//                                 previous alpha_x
 //   vecR   [Q][4][ld]      Real   p, alpha_x, x0, next starting guess (stream precision);
 //                                 then theta [ld]
 //   state  [Q]             SolveState
@@ -39,6 +41,7 @@ constexpr int kPartScal = 4;
 constexpr int kVec64 = 9;
 constexpr int kRedTile = 128;  // elements per block of the partial reduction and CG update
 constexpr int kBpart = 4;      // per-block shares: w . r, S . r, r . r, spare
+constexpr int kDpart = 4;      // doubles per chunk's share of r . A r: one 32-byte sector each
 constexpr int kVecR = 4;
 constexpr int kSegSums = 6;   // per-row-segment sums of the row kernels (the forward SDE's
                               // rows use all six, the driftless ones the first four)
@@ -67,6 +70,15 @@ struct Layout {
     size_t off_tape_w, off_tape_Y, off_tape_v, off_tape_s, off_adj_v, total_adjoint;
     int seg_vpt, nseg, GP, mom_vm, mom_tiles, row_blocks, mv_rows, mv_stages, red_groups, nblk;
     size_t mv_smem;
+    // CG: row chunks per query of the product, lanes per row of partials and tiles of phase
+    // B; the loop's ring (rows per stage, stages, rows in all), whether it holds a CTA's rows for the
+    // whole loop, bytes of its operand (0 or 1 row), shared sums and shared memory; cg_ok:
+    // the loop covers this shape
+    int mv_mode, Gc, cg_lpr, cg_nblk, cg_rows, cg_stages, cg_ring, cg_res, cg_op, cg_both, cg_ok;
+    size_t cg_smem;
+    // the pass in three launches (fbsde_cg3.cuh) instead, with its own team geometry and ring
+    int cg3, c3_tw, c3_vpt, c3_teams, c3_rows, c3_stages;
+    size_t c3_smem;
     // fused per-level step (FP32 rows of at most kStepMaxLd floats): rows per stage, threads
     // per row, chunks per thread in the row pass, column-pass row groups, shared memory
     int fused, st_R, st_T, st_vm1, st_tpr, st_RG, st_vm3, st_vm, st_nslot, GS, Gs;
@@ -111,7 +123,12 @@ struct Params {
     double *vec64;
     void *vecR;
     SolveState *st;
-    double *bpart;  // [Q][nblk][kBpart] per-block shares of the CG dot products
+    double *dpart;   // [Q][Gc][kDpart] the product chunks' shares of r . A r (in segp, free during the CG)
+    double *bpart;   // [Q][nblk3][kBpart] shares of the pass in three launches
+    int nblk3;
+    unsigned int *bar;   // grid barrier of the CG loop (in bpart, which it does not use)
+    int part_vecs;       // vectors per partial: 3 (moments) or 1 (product)
+    int cg_teams, cg_lpr, cg_rows, cg_stages, cg_ring, cg_res, cg_op, cg_both;
     // tape of the primal for the reverse sweep (null when not recording)
     void *tape_w;
     double *tape_Y, *tape_v, *tape_s, *adj_v;
@@ -137,12 +154,17 @@ template <typename Real> struct Launch {
     static cudaError_t sde_rows(const Params &p, const Layout &L, int k, const void *src,
                                 cudaStream_t s);
     static cudaError_t sde_rho(const Params &p, const Layout &L, cudaStream_t s);
-    static cudaError_t reduce(const Params &p, const Layout &L, int nvec, int dst0, int skip_done,
+    static cudaError_t reduce(const Params &p, const Layout &L, int nvec, int dst0,
                               cudaStream_t s);
     static cudaError_t matvec(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t moments_finalize(const Params &p, const Layout &L, int warm, cudaStream_t s);
-    static cudaError_t cg_update(const Params &p, const Layout &L, cudaGraphConditionalHandle h,
+    static cudaError_t cg_tile(const Params &p, const Layout &L, cudaGraphConditionalHandle h,
                                int use_h, cudaStream_t s);
+    // the pass in three launches (0: product, 1: reduction, 2: updates), FP32 only
+    static cudaError_t cg3(const Params &p, const Layout &L, int kernel, cudaGraphConditionalHandle h,
+                           int use_h, cudaStream_t s);
+    static bool cg_loop_fits(const Layout &L);   // on the current device
+    static cudaError_t cg_loop(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t cg_post(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t cg_reset(const Params &p, cudaGraphConditionalHandle h, cudaStream_t s);
     static cudaError_t trace_forward(const Params &p, const Layout &L, cudaStream_t s);

@@ -11,9 +11,9 @@
 //   k_moments              streaming weighted column sums of the particle rows;
 //   k_matvec               the matrix-free product of the regression operator (a team
 //                          of warps per row: dot product, then the weighted row sum);
-//   k_reduce_partials      fixed-order compensated sum of the per-CTA partial vectors,
-//                          and in the CG the operator's FP64 epilogue (tiles of 128);
-//   k_cg_update            one CG pass of the d-vectors, tiles of 128 elements per block;
+//   k_cg_loop, k_cg_tile   the conjugate gradients (fbsde_cg.cuh);
+//   k_reduce_partials      fixed-order compensated sum of the per-CTA partial vectors
+//                          (tiles of 128);
 //   k_moments_finalize, k_cg_post, k_setup
 //                          one CTA per query: FP64 d-vector algebra of the regression.
 #pragma once
@@ -173,6 +173,13 @@ template <typename Real> __device__ __forceinline__ Chunk<Real> ldg_chunk(const 
 {
     Chunk<Real> c;
     *reinterpret_cast<int4 *>(c.v) = __ldg(reinterpret_cast<const int4 *>(p));
+    return c;
+}
+// Through L2 only (values that other SMs wrote during this launch).
+template <typename Real> __device__ __forceinline__ Chunk<Real> ldcg_chunk(const Real *p)
+{
+    Chunk<Real> c;
+    *reinterpret_cast<int4 *>(c.v) = __ldcg(reinterpret_cast<const int4 *>(p));
     return c;
 }
 template <typename Real> __device__ __forceinline__ void st_chunk(Real *p, const Chunk<Real> &c)
@@ -462,7 +469,7 @@ template <typename Real> struct WS {
     }
     __device__ __forceinline__ Real *part(int s, int g, int v) const
     {
-        return reinterpret_cast<Real *>(p.part) + (((size_t)s * p.G + g) * kPartVecs + v) * p.ld;
+        return reinterpret_cast<Real *>(p.part) + (((size_t)s * p.G + g) * p.part_vecs + v) * p.ld;
     }
     __device__ __forceinline__ double *spart(int s, int b) const
     {
@@ -922,11 +929,7 @@ __global__ void __launch_bounds__(256) k_moments(Params p)
 // element t in group order.  With FP32 partials every addition is compensated (Neumaier
 // 1974): the running sum and its error term stay in FP32 and only the final s + c is
 // widened to FP64.  FP64 partials are added in FP64.
-//   cg_mode = 0: vectors 0..nvec-1 into v64 slots dst0..
-//   cg_mode = 1: the product of the CG pass (queries already converged skip):
-//       w = sum / W - S (S . r) + lambda r   (Gamma_c r + lambda r, Eq. 3.19's operator)
-//     into slot 5 and this block's share of w . r into bpart; every block of k_cg_update
-//     adds the shares and derives the pass's scalars from them.
+// Vectors 0..nvec-1 go into the v64 slots dst0..
 // Grid (nblk, Q), nblk = ceil(ld / kRedTile).
 template <typename Real> struct RedAcc {
     double s;
@@ -974,23 +977,34 @@ template <typename Real> __device__ __forceinline__ Quad<Real> ld_quad(const Rea
     return q;
 }
 
+template <typename Real> __device__ __forceinline__ Quad<Real> ldcg_quad(const Real *p)
+{
+    Quad<Real> q;
+    if constexpr (sizeof(Real) == 4) {
+        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
+        q.v[0] = t.x; q.v[1] = t.y; q.v[2] = t.z; q.v[3] = t.w;
+    } else {
+        const double2 a = __ldcg(reinterpret_cast<const double2 *>(p));
+        const double2 b = __ldcg(reinterpret_cast<const double2 *>(p + 2));
+        q.v[0] = a.x; q.v[1] = a.y; q.v[2] = b.x; q.v[3] = b.y;
+    }
+    return q;
+}
+
 template <typename Real>
-__global__ void __launch_bounds__(512) k_reduce_partials(Params p, int nvec, int dst0, int cg_mode)
+__global__ void __launch_bounds__(512) k_reduce_partials(Params p, int nvec, int dst0)
 {
     using Acc = RedAcc<Real>;
     using Lo = decltype(Acc{}.lo());
     constexpr int kB = 8;  // loads in flight per lane
     __shared__ Real sh_s[16][kRedTile];
     __shared__ Lo sh_c[16][kRedTile];
-    __shared__ double sh_w[4];
     const int s = blockIdx.y;
-    SolveState &st = p.st[s];
-    if (cg_mode && st.done) return;
     const int lane = threadIdx.x & 31, gg = threadIdx.x >> 5, GR = blockDim.x >> 5;
     const int e0 = blockIdx.x * kRedTile + 4 * lane;  // first element of this lane
     const bool in = e0 < p.ld;                        // ld is a multiple of 4
     const WS<Real> ws(p);
-    const size_t stride = (size_t)kPartVecs * p.ld * GR;   // between this group's partials
+    const size_t stride = (size_t)p.part_vecs * p.ld * GR;   // between this group's partials
     for (int v = 0; v < nvec; ++v) {
         Acc acc[4];
 #pragma unroll
@@ -1023,26 +1037,10 @@ __global__ void __launch_bounds__(512) k_reduce_partials(Params p, int nvec, int
             tot.init();
             for (int k = 0; k < GR; ++k) tot.merge(sh_s[k][t], sh_c[k][t]);
             const double sum = tot.value();
-            if (!cg_mode) {
-                if (i < p.ld) ws.v64(s, dst0 + v)[i] = sum;
-            } else {
-                double wr = 0.0;
-                if (i < p.ld) {
-                    const double ri = ws.v64(s, 1)[i];
-                    const double wi = sum * st.invW - ws.v64(s, 3)[i] * st.sp + st.lambda * ri;
-                    ws.v64(s, 5)[i] = wi;
-                    wr = wi * ri;
-                }
-#pragma unroll
-                for (int o = 16; o; o >>= 1) wr += __shfl_xor_sync(0xffffffffu, wr, o);
-                if (lane == 0) sh_w[t >> 5] = wr;
-            }
+            if (i < p.ld) ws.v64(s, dst0 + v)[i] = sum;
         }
         __syncthreads();
     }
-    if (!cg_mode) return;
-    if (threadIdx.x == 0)   // the next kernel boundary makes the shares visible
-        p.bpart[((size_t)s * p.nblk + blockIdx.x) * kBpart] = ((sh_w[0] + sh_w[1]) + sh_w[2]) + sh_w[3];
 }
 
 // ---------------------------------------------------------------------------
@@ -1103,6 +1101,7 @@ __global__ void __launch_bounds__(kFinThreads) k_setup(Params p, const double *x
         st.gx0 = g_value(p, phi);
         st.yref = st.gx0;
         p.st[s] = st;
+        if (s == 0) *p.bar = 0u;   // the CG loop's grid barrier
     }
 }
 
@@ -1185,174 +1184,6 @@ __global__ void __launch_bounds__(kFinThreads) k_moments_finalize(Params p, int 
         st.sp = a2[2];
         st.iters = 0;
         st.done = (a2[1] <= p.cg_tol2 * a2[0]) ? 1 : 0;
-    }
-}
-
-// Four consecutive values at a 16-byte aligned address (two 16-byte accesses for doubles,
-// one for floats).
-__device__ __forceinline__ void ld4(double (&v)[4], const double *q)
-{
-    const double2 a = *reinterpret_cast<const double2 *>(q);
-    const double2 b = *reinterpret_cast<const double2 *>(q + 2);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-__device__ __forceinline__ void st4(double *q, const double (&v)[4])
-{
-    *reinterpret_cast<double2 *>(q) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2 *>(q + 2) = make_double2(v[2], v[3]);
-}
-__device__ __forceinline__ void st4(float *q, const float (&v)[4])
-{
-    *reinterpret_cast<float4 *>(q) = make_float4(v[0], v[1], v[2], v[3]);
-}
-
-// One pass of the CG iteration of Chronopoulos and Gear (1989), the form of conjugate
-// gradients with a single reduction phase per iteration.  The product w = A r and the
-// shares of delta = w . r come from k_reduce_partials; every block adds the shares in
-// the same order and derives the pass's scalars (gamma = r . r):
-//   t = 0: beta = 0, a = gamma / delta;
-//   t > 0: beta = gamma / gamma_prev, a = gamma / (delta - beta gamma / a_prev),
-// then
-//   p = r + beta p,  s = w + beta s (= A p),  x += a p,  r -= a s,
-// one warp per tile of kRedTile elements (four consecutive elements per lane), with the
-// tile's shares of S . r and r . r for the next pass.  The last block of the query to
-// finish (arrival counter) adds those shares, stores the new state and tests convergence;
-// a query that is done stays done, so every block of a launch sees the same state.  Each
-// FP64 warp instruction occupies the SM's FP64 pipe for many cycles on this part, so the
-// scalar work is done once per query (in the reduction) rather than once per block.  In a
-// CUDA graph (use_h = 1) the last query to finish sets the while-loop condition: 1 while
-// some query has not converged and fewer than cg_max_iter passes ran (with one query,
-// its last block does so without the second arrival).  Grid (nblk, Q).
-template <typename Real>
-__global__ void __launch_bounds__(32) k_cg_update(Params p, cudaGraphConditionalHandle h, int use_h)
-{
-    const int s = blockIdx.y, lane = threadIdx.x;
-    SolveState &st = p.st[s];
-    bool global_arrive = false;
-    if (st.done) {
-        global_arrive = blockIdx.x == 0;   // one block answers for a finished query
-    } else {
-        const WS<Real> ws(p);
-        double *x = ws.v64(s, 0), *r = ws.v64(s, 1), *pp = ws.v64(s, 2), *S = ws.v64(s, 3),
-               *w = ws.v64(s, 5), *sv = ws.v64(s, 7);
-        Real *rR = ws.vR(s, 0);
-        double *bp = p.bpart + (size_t)s * p.nblk * kBpart;
-        const int t = st.iters;
-        const double gam = st.rr;
-        const int i0 = blockIdx.x * kRedTile + 4 * lane;
-        const bool in = i0 < p.ld;   // ld is a multiple of 4
-        // every value of the lane's four elements is loaded first, before the pass's scalars
-        // are derived and before the first store (the vectors may alias as far as the
-        // compiler can tell, so it would not move a later element's loads above a store)
-        double rv[4], wv[4], pv[4], svv[4], xv[4], Sv[4];
-        if (in) {
-            ld4(rv, r + i0);
-            ld4(wv, w + i0);
-            ld4(xv, x + i0);
-            ld4(Sv, S + i0);
-            if (t > 0) {
-                ld4(pv, pp + i0);
-                ld4(svv, sv + i0);
-            }
-        }
-        double dl = 0.0;   // delta = w . r: the shares in a fixed order, the same in every block
-        for (int b = lane; b < p.nblk; b += 32) dl += __ldcg(bp + (size_t)b * kBpart);
-#pragma unroll
-        for (int o = 16; o; o >>= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
-        double beta = 0.0, den = dl;
-        if (t > 0) {
-            beta = gam / st.rr_prev;
-            den = dl - beta * gam / st.cg_alpha;
-        }
-        const double a = gam / den;
-        const int ok = (den > 0.0 && isfinite(a)) ? 1 : 0;
-        double sr = 0.0, rr = 0.0;
-        if (ok && in) {
-            Real rn4[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const double pi = t > 0 ? rv[e] + beta * pv[e] : rv[e];
-                const double si = t > 0 ? wv[e] + beta * svv[e] : wv[e];
-                pv[e] = pi;
-                svv[e] = si;
-                xv[e] += a * pi;
-                const double rn = rv[e] - a * si;
-                rv[e] = rn;
-                rn4[e] = (Real)rn;
-                sr += Sv[e] * rn;
-                rr += rn * rn;
-            }
-            st4(pp + i0, pv);
-            st4(sv + i0, svv);
-            st4(x + i0, xv);
-            st4(r + i0, rv);
-            st4(rR + i0, rn4);
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            sr += __shfl_xor_sync(0xffffffffu, sr, o);
-            rr += __shfl_xor_sync(0xffffffffu, rr, o);
-        }
-        int last = 0;
-        if (lane == 0) {
-            bp[(size_t)blockIdx.x * kBpart + 1] = sr;
-            bp[(size_t)blockIdx.x * kBpart + 2] = rr;
-            __threadfence();
-            last = atomicAdd(&st.arrive_q, 1) == p.nblk - 1;
-        }
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (last) {
-            __threadfence();
-            double c0 = 0.0, c1 = 0.0;
-            for (int b = lane; b < p.nblk; b += 32) {
-                c0 += __ldcg(bp + (size_t)b * kBpart + 1);
-                c1 += __ldcg(bp + (size_t)b * kBpart + 2);
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-                c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            }
-            if (lane == 0) {
-                st.arrive_q = 0;
-                if (!ok) {  // breakdown: keep the current iterate
-                    st.done = 1;
-                    if (!(gam <= p.cg_tol2 * st.rhs2) && st.status == 0) st.status = FBSDE_ERR_CG;
-                } else {
-                    st.rr_prev = gam;
-                    st.cg_alpha = a;
-                    st.rr = c1;
-                    st.sp = c0;
-                    st.iters = t + 1;
-                    st.cg_total += 1;
-                    if (c1 <= p.cg_tol2 * st.rhs2) {
-                        st.done = 1;
-                    } else if (t + 1 >= p.cg_max_iter) {
-                        st.done = 1;
-                        st.cg_exhausted += 1;
-                        if (st.status == 0) st.status = FBSDE_ERR_CG;
-                    }
-                }
-                global_arrive = true;
-            }
-        }
-    }
-    if (use_h && global_arrive && lane == 0) {
-        bool last_q = true;   // one query: its last block is the last arrival
-        if (p.Q > 1) {
-            __threadfence();
-            last_q = atomicAdd(&p.st[0].arrive, 1) == p.Q - 1;
-        }
-        if (last_q) {
-            if (p.Q > 1) __threadfence();
-            p.st[0].arrive = 0;
-            const int count = ++p.st[0].loop_iter;
-            bool active = false;
-            for (int q2 = 0; q2 < p.Q && !active; ++q2)
-                active = *reinterpret_cast<volatile int *>(&p.st[q2].done) == 0;
-            if (count >= p.cg_max_iter) active = false;
-            cudaGraphSetConditional(h, active ? 1u : 0u);
-        }
     }
 }
 

@@ -1,6 +1,8 @@
 // fbsde_launch.cuh -- host launchers of the kernels for one stream precision.
 #pragma once
 #include "fbsde_adjoint.cuh"
+#include "fbsde_cg.cuh"
+#include "fbsde_cg3.cuh"
 #include "fbsde_kernels.cuh"
 #include "fbsde_matvec.cuh"
 #include "fbsde_sde.cuh"
@@ -191,36 +193,39 @@ cudaError_t Launch<Real>::step(const Params &p, const Layout &L, cudaStream_t s)
 
 template <typename Real>
 cudaError_t Launch<Real>::reduce(const Params &p, const Layout &L, int nvec, int dst0,
-                                 int skip_done, cudaStream_t s)
+                                 cudaStream_t s)
 {
-    dev::k_reduce_partials<Real><<<dim3(L.nblk, L.Q), 32 * L.red_groups, 0, s>>>(p, nvec, dst0,
-                                                                                 skip_done);
+    dev::k_reduce_partials<Real><<<dim3(L.nblk, L.Q), 32 * L.red_groups, 0, s>>>(p, nvec, dst0);
     return cudaGetLastError();
 }
 
-template <typename Real, int VPT, bool WIDE>
+template <typename Real, int VPT, int MODE>
 static cudaError_t launch_matvec(const Params &p, const Layout &L, cudaStream_t s)
 {
-    cudaError_t e = set_smem(dev::k_matvec<Real, VPT, WIDE>, L.mv_smem);
+    cudaError_t e = set_smem(dev::k_matvec<Real, VPT, MODE>, L.mv_smem);
     if (e != cudaSuccess) return e;
-    dev::k_matvec<Real, VPT, WIDE>
-        <<<dim3(L.G, L.Q), 32 * (1 + L.teams * L.team_warps), L.mv_smem, s>>>(p);
+    dev::k_matvec<Real, VPT, MODE>
+        <<<dim3(L.Gc, L.Q), 32 * (1 + L.teams * L.team_warps), L.mv_smem, s>>>(p);
     return cudaGetLastError();
 }
 
 template <typename Real>
 cudaError_t Launch<Real>::matvec(const Params &p, const Layout &L, cudaStream_t s)
 {
-    const bool wide = 32 * (1 + L.teams * L.team_warps) > 352;
     switch (L.vpt) {
-    case 1: return launch_matvec<Real, 1, false>(p, L, s);
-    case 2: return launch_matvec<Real, 2, false>(p, L, s);
-    case 4: return launch_matvec<Real, 4, false>(p, L, s);
-    case 8: return wide ? launch_matvec<Real, 8, true>(p, L, s)
-                        : launch_matvec<Real, 8, false>(p, L, s);
+    case 1: return launch_matvec<Real, 1, dev::kMvHold>(p, L, s);
+    case 2: return launch_matvec<Real, 2, dev::kMvHold>(p, L, s);
+    case 4: return launch_matvec<Real, 4, dev::kMvHold>(p, L, s);
+    case 8:
+        switch (L.mv_mode) {
+        case dev::kMvHold: return launch_matvec<Real, 8, dev::kMvHold>(p, L, s);
+        case dev::kMvPair: return launch_matvec<Real, 8, dev::kMvPair>(p, L, s);
+        case dev::kMvWide: return launch_matvec<Real, 8, dev::kMvWide>(p, L, s);
+        }
+        return cudaErrorInvalidValue;
     case 16:   // FP64 rows of 8193 to 10240 values: teams of 9 or 10 warps
         if constexpr (sizeof(Real) == 8) {
-            if (!wide) return launch_matvec<Real, 16, false>(p, L, s);
+            if (L.team_warps <= 10) return launch_matvec<Real, 16, dev::kMvPair>(p, L, s);
         }
         return cudaErrorInvalidValue;
     }
@@ -236,11 +241,104 @@ cudaError_t Launch<Real>::moments_finalize(const Params &p, const Layout &L, int
 }
 
 template <typename Real>
-cudaError_t Launch<Real>::cg_update(const Params &p, const Layout &L, cudaGraphConditionalHandle h,
-                                    int use_h, cudaStream_t s)
+cudaError_t Launch<Real>::cg_tile(const Params &p, const Layout &L, cudaGraphConditionalHandle h,
+                                  int use_h, cudaStream_t s)
 {
-    dev::k_cg_update<Real><<<dim3(L.nblk, L.Q), 32, 0, s>>>(p, h, use_h);
+    dev::k_cg_tile<Real><<<dim3(L.cg_nblk, L.Q), dev::kCgThreads, 0, s>>>(p, h, use_h);
     return cudaGetLastError();
+}
+
+template <int VPT, bool WIDE>
+static cudaError_t launch_product(const Params &p, const Layout &L, cudaStream_t s)
+{
+    cudaError_t e = set_smem(dev::k_product<float, VPT, WIDE>, L.c3_smem);
+    if (e != cudaSuccess) return e;
+    dev::k_product<float, VPT, WIDE>
+        <<<dim3(L.G, L.Q), 32 * (1 + L.c3_teams * L.c3_tw), L.c3_smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t Launch<Real>::cg3(const Params &p0, const Layout &L, int kernel,
+                              cudaGraphConditionalHandle h, int use_h, cudaStream_t s)
+{
+    if constexpr (sizeof(Real) != sizeof(float)) {
+        return cudaErrorInvalidValue;
+    } else {
+        Params p = p0;
+        p.G = L.G;
+        p.part_vecs = kPartVecs;
+        p.team_warps = L.c3_tw;
+        p.mv_rows = L.c3_rows;
+        p.mv_stages = L.c3_stages;
+        const dim3 tiles(L.nblk, L.Q);
+        switch (kernel) {
+        case 0:
+            switch (L.c3_vpt) {
+            case 1: return launch_product<1, false>(p, L, s);
+            case 2: return launch_product<2, false>(p, L, s);
+            case 4: return launch_product<4, false>(p, L, s);
+            case 8:
+                return 32 * (1 + L.c3_teams * L.c3_tw) > 352 ? launch_product<8, true>(p, L, s)
+                                                             : launch_product<8, false>(p, L, s);
+            }
+            return cudaErrorInvalidValue;
+        case 1: dev::k_product_reduce<float><<<tiles, 32 * L.red_groups, 0, s>>>(p); break;
+        case 2: dev::k_cg_update<float><<<tiles, 32, 0, s>>>(p, h, use_h); break;
+        default: return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+    }
+}
+
+// SMs of the current device, 0 without cooperative launches.
+static int coop_sms()
+{
+    int dev = 0, n = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return n;
+}
+
+template <typename Real>
+static void *cg_loop_kernel(const Layout &L)
+{
+    switch (L.vpt) {
+    case 1: return reinterpret_cast<void *>(dev::k_cg_loop<Real, 1, 512, true>);
+    case 2: return reinterpret_cast<void *>(dev::k_cg_loop<Real, 2, 512, true>);
+    case 4: return reinterpret_cast<void *>(dev::k_cg_loop<Real, 4, 512, true>);
+    case 8:
+        return L.mv_mode == dev::kMvHold
+                   ? reinterpret_cast<void *>(dev::k_cg_loop<Real, 8, 352, true>)
+                   : reinterpret_cast<void *>(dev::k_cg_loop<Real, 8, 352, false>);
+    }
+    return nullptr;
+}
+
+// A layout that keeps one chunk per CTA in shared memory needs that many CTAs at once.
+template <typename Real> bool Launch<Real>::cg_loop_fits(const Layout &L)
+{
+    if (!L.cg_ok || !cg_loop_kernel<Real>(L)) return false;
+    const int sms = coop_sms();
+    return sms > 0 && (!L.cg_res || (long long)L.Q * L.Gc <= sms);
+}
+
+template <typename Real>
+cudaError_t Launch<Real>::cg_loop(const Params &p, const Layout &L, cudaStream_t s)
+{
+    void *k = cg_loop_kernel<Real>(L);
+    const int sms = coop_sms();
+    if (!k || sms < 1) return cudaErrorNotSupported;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)L.cg_smem);
+    if (e != cudaSuccess) return e;
+    const long long work = (long long)L.Q * std::max(L.Gc, L.cg_nblk);
+    Params q = p;
+    void *args[] = {&q};
+    return cudaLaunchCooperativeKernel(k, dim3((unsigned)std::min<long long>(sms, work)),
+                                       dim3(L.vpt == 8 ? 352 : 512), args, L.cg_smem, s);
 }
 
 template <typename Real>

@@ -1,5 +1,5 @@
 // fbsde_matvec.cuh -- the matrix-free product of the regression operator (the dominant
-// kernel of a solve), fed by bulk copies (TMA) through an mbarrier-synchronised
+// work of a solve), fed by bulk copies (TMA) through an mbarrier-synchronised
 // shared-memory ring.  Included after fbsde_kernels.cuh.
 #pragma once
 #include "fbsde_kernels.cuh"
@@ -92,21 +92,337 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
 }
 
 // ---------------------------------------------------------------------------
-// Matrix-free product of the regression (Sec. 2.4, Steps 1 and 2) on the centred
-// operator: partial_g = sum_{j in CTA g} w_j (D_j . v) D_j with v = vR(s, 0).
-// Warp 0 is the producer: one lane streams the CTA's rows, mv_rows consecutive rows
-// (one contiguous block) per stage, into a ring of mv_stages shared-memory stages
-// with cp.async.bulk, completion counted on the stage's "full" mbarrier.  The other
-// warps form nteams consumer teams of team_warps warps; a team owns one row at a time:
-// dot product from shared memory, team sum (warp butterfly + one named barrier),
-// then the weighted row sum into register accumulators.  Each consumer warp arrives
-// on the stage's "empty" mbarrier when done, which lets the producer refill it.
+// Matrix-free product of the regression (Sec. 2.4, Steps 1 and 2) on the centred operator:
+// for one chunk g of a query's rows, partial_g = sum_j w_j (D_j . r) D_j and the share
+// sum_j w_j (D_j . r)^2 of r^T A r, r = vR(s, 0).  The rows reach shared memory by bulk
+// copies; nteams teams of tw warps take one row at a time: dot product, team sum (warp
+// butterfly + one named barrier), then the weighted row sum into register accumulators.
+// The team of a row is its index in the chunk modulo nteams, so the sums do not depend on
+// how the rows are staged; k_matvec (one launch per product) and k_cg_loop (the whole CG
+// in one launch) run these functions on the same chunks and give the same bits.
 // ---------------------------------------------------------------------------
-template <typename Real, int VPT, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? 544 : (VPT >= 8 ? 352 : 288), 1) k_matvec(Params p)
+struct MvTeam {
+    int tw, nteams, tthreads, team, tl, wt, lane, nch;
+    __device__ __forceinline__ MvTeam(int tw_, int nteams_, int nch_)   // consumers: warps 1..
+        : tw(tw_), nteams(nteams_), tthreads(32 * tw_), lane(threadIdx.x & 31), nch(nch_)
+    {
+        const int ct = (int)threadIdx.x - 32;
+        team = ct / tthreads;
+        tl = ct - team * tthreads;
+        wt = tl >> 5;
+    }
+};
+
+// Dot product and weighted sum of 16-byte chunks; FP32 as pairs (one packed instruction for
+// two fused multiply-adds).
+template <typename Real> struct DotAcc;
+template <> struct DotAcc<double> {
+    double s;
+    __device__ __forceinline__ void init() { s = 0.0; }
+    __device__ __forceinline__ void add(const Chunk<double> &a, const Chunk<double> &b)
+    {
+        s = fma(a.v[0], b.v[0], s);
+        s = fma(a.v[1], b.v[1], s);
+    }
+    __device__ __forceinline__ double sum() const { return s; }
+};
+template <> struct DotAcc<float> {
+    float2 s;
+    __device__ __forceinline__ void init() { s = make_float2(0.f, 0.f); }
+    __device__ __forceinline__ void add(const Chunk<float> &a, const Chunk<float> &b)
+    {
+        s = __ffma2_rn(make_float2(a.v[0], a.v[1]), make_float2(b.v[0], b.v[1]), s);
+        s = __ffma2_rn(make_float2(a.v[2], a.v[3]), make_float2(b.v[2], b.v[3]), s);
+    }
+    __device__ __forceinline__ float sum() const { return s.x + s.y; }
+};
+__device__ __forceinline__ void chunk_axpy(Chunk<double> &y, double a, const Chunk<double> &x)
+{
+    y.v[0] = fma(a, x.v[0], y.v[0]);
+    y.v[1] = fma(a, x.v[1], y.v[1]);
+}
+__device__ __forceinline__ void chunk_axpy(Chunk<float> &y, float a, const Chunk<float> &x)
+{
+    const float2 aa = make_float2(a, a);
+    const float2 l = __ffma2_rn(aa, make_float2(x.v[0], x.v[1]), make_float2(y.v[0], y.v[1]));
+    const float2 h = __ffma2_rn(aa, make_float2(x.v[2], x.v[3]), make_float2(y.v[2], y.v[3]));
+    y.v[0] = l.x;
+    y.v[1] = l.y;
+    y.v[2] = h.x;
+    y.v[3] = h.y;
+}
+
+// NR rows at a time (1 or 2): t = row . r, acc += w t row in row order; the team's first
+// thread adds w t^2 to dacc.  rel0, rel1: "empty" barriers of the stages whose last rows
+// these are (or null); with the rows held in registers they are released before the
+// butterfly, which leaves the ring more bytes in flight.  Two rows share the latency of the loads, the butterfly and the
+// team's barrier: the butterfly's first step leaves one row's sums in each half of the warp,
+// so its other steps add both at once.  Each row's sum has the same bits either way.
+// kReread: the thread's chunks of the row are read from shared memory again for the weighted
+// sum (teams of more than 10 warps, or 16 chunks per thread, whose registers are short); with
+// 16 the operand too is read from memory for every row.
+template <typename Real, int VPT, bool kReread, int NR>
+__device__ __forceinline__ void mv_rows(const Real *const (&row)[NR], const Real (&w)[NR],
+                                        const Real *opmem, const Chunk<Real> (&pc)[VPT],
+                                        Chunk<Real> (&acc)[VPT], RedAcc<Real> &dacc, const MvTeam &m,
+                                        Real *slots, int &phase, uint64_t *rel0, uint64_t *rel1)
+{
+    constexpr int E = Chunk<Real>::E;
+    constexpr bool kOpMem = VPT > 8;
+    auto release = [&]() {
+        __syncwarp();
+        if (m.lane == 0) {
+            if (rel0) mbar_arrive(rel0);
+            if (rel1) mbar_arrive(rel1);
+        }
+    };
+    constexpr int kHeld = kReread ? 1 : VPT;
+    Chunk<Real> dl[NR][kHeld];
+    DotAcc<Real> ta[NR];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) ta[n].init();
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        // past the row's end: its last chunk, with a zero operand (and sums never stored)
+        const int c = m.tl + m.tthreads * v, cc = min(c, m.nch - 1);
+        Chunk<Real> o;
+        if (!kOpMem) {
+            o = pc[v];
+        } else {
+            if (c < m.nch) o = ldg_chunk(opmem + c * E);
+            else zero(o);
+        }
+#pragma unroll
+        for (int n = 0; n < NR; ++n) {
+            Chunk<Real> &x = dl[n][kReread ? 0 : v];
+            x = ld_chunk(row[n] + cc * E);
+            ta[n].add(x, o);
+        }
+    }
+    Real t[NR];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) t[n] = ta[n].sum();
+    if (!kReread) release();   // the rows are in registers
+    if constexpr (NR == 2) {
+        const bool hi = m.lane & 16;
+        Real keep = hi ? t[1] : t[0];
+        const Real give = hi ? t[0] : t[1];
+        keep += __shfl_xor_sync(0xffffffffu, give, 16);
+#pragma unroll
+        for (int o = 8; o; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+        if (m.tw == 1) {
+            const Real other = __shfl_xor_sync(0xffffffffu, keep, 16);
+            t[0] = hi ? other : keep;
+            t[1] = hi ? keep : other;
+        } else {
+            Real *sl = slots + (size_t)(m.team * 2 + phase) * 32;
+            if ((m.lane & 15) == 0) sl[2 * m.wt + (hi ? 1 : 0)] = keep;
+        }
+    } else {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+        if (m.tw > 1) {
+            Real *sl = slots + (size_t)(m.team * 2 + phase) * 32;
+            if (m.lane == 0) sl[2 * m.wt] = t[0];
+        }
+    }
+    if (m.tw > 1) {
+        const Real *sl = slots + (size_t)(m.team * 2 + phase) * 32;
+        bar_named(1 + m.team, m.tthreads);
+#pragma unroll
+        for (int n = 0; n < NR; ++n) t[n] = Real(0);
+        for (int w2 = 0; w2 < m.tw; ++w2) {
+#pragma unroll
+            for (int n = 0; n < NR; ++n) t[n] += sl[2 * w2 + n];
+        }
+        phase ^= 1;
+    }
+#pragma unroll
+    for (int n = 0; n < NR; ++n) {
+        const Real coef = w[n] * t[n];
+        if (m.tl == 0) dacc.add(coef * t[n]);   // compensated in FP32: no FP64 in the row loop
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            if (kReread) dl[n][0] = ld_chunk(row[n] + min(m.tl + m.tthreads * v, m.nch - 1) * E);
+            chunk_axpy(acc[v], coef, dl[n][kReread ? 0 : v]);
+        }
+    }
+    if (kReread) release();
+}
+
+// How a team of 8 chunks per thread walks its rows (4 and fewer: always held, in pairs):
+//   kMvHold  several teams share the rows: one row at a time, held in registers, its stage
+//            released before the butterfly (d = 1000, M = 4096, 64 queries: 169 us a product,
+//            184 us in pairs, whose two stages leave the ring fewer bytes in flight);
+//   kMvPair  one team for all rows: two at a time, read again for the weighted sum, so that
+//            one butterfly and one barrier serve both (d = 10^4, M = 16384, 16 queries:
+//            1375 us a product, 1540 us one at a time: the chain of a row's steps bounds it);
+//   kMvWide  as kMvPair with teams of 11 to 16 warps.
+enum MvMode { kMvHold = 0, kMvPair = 1, kMvWide = 2 };
+
+// Position of a consumer in the ring of row stages.
+struct MvRing {
+    int slot, par, S, R;
+    __device__ __forceinline__ void next()
+    {
+        if (++slot == S) {
+            slot = 0;
+            par ^= 1;
+        }
+    }
+};
+
+// The consumers' part of one chunk, rows [r0, r1): its stages of R rows (a multiple of the
+// teams) from the ring, released after use unless they stay (release = false).  wv: the
+// weights from row r0 on.  kPair: two rows of a team at a time (of two stages where a stage
+// holds one row per team).
+template <typename Real, int VPT, bool kReread, bool kPair>
+__device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real *wv,
+                                         const Real *opmem, const Chunk<Real> (&pc)[VPT],
+                                         Chunk<Real> (&acc)[VPT], RedAcc<Real> &dacc, const MvTeam &m,
+                                         const Real *ring, uint64_t *full, uint64_t *empty,
+                                         MvRing &rg, bool release, Real *slots, int &phase,
+                                         bool &timed_out)
+{
+    const size_t ld = (size_t)m.nch * Chunk<Real>::E;
+    const int nrows = (int)(r1 - r0), nt = m.nteams;
+    const bool across = kPair && rg.R == nt;
+    auto one = [&](const Real *p0, Real w0, uint64_t *rel) {
+        const Real *const row[1] = {p0};
+        const Real w[1] = {w0};
+        mv_rows<Real, VPT, kReread, 1>(row, w, opmem, pc, acc, dacc, m, slots, phase, rel, nullptr);
+    };
+    auto none = [&](uint64_t *rel0, uint64_t *rel1) {   // stages without a row for this team
+        if (m.lane == 0) {
+            if (rel0) mbar_arrive(rel0);
+            if (rel1) mbar_arrive(rel1);
+        }
+    };
+    // the weights of the team's next two rows, requested one step ahead of their use
+    auto weight = [&](int j) { return j < nrows ? wv[j] : Real(0); };
+    Real n0 = weight(m.team), n1 = weight(m.team + nt);
+    for (int base = 0; base < nrows;) {
+        const int a = rg.slot, rows = min(rg.R, nrows - base);
+        const Real *buf = ring + (size_t)a * rg.R * ld;
+        uint64_t *ea = release ? &empty[a] : nullptr;
+        if (across) {
+            const int j = base + m.team, j2 = j + nt;
+            const bool two = base + nt < nrows;   // this stage and the next
+            const Real w0 = n0, w1 = n1;
+            n0 = weight(j + 2 * nt);
+            n1 = weight(j + 3 * nt);
+            mbar_wait_or_flag(&full[a], (uint32_t)rg.par, timed_out);
+            rg.next();
+            const int b = rg.slot;
+            if (two) {
+                mbar_wait_or_flag(&full[b], (uint32_t)rg.par, timed_out);
+                rg.next();
+            }
+            uint64_t *eb = release && two ? &empty[b] : nullptr;
+            const Real *p0 = buf + (size_t)m.team * ld;
+            const Real *p1 = ring + ((size_t)b * rg.R + m.team) * ld;
+            if constexpr (kPair) {
+                if (j2 < nrows) {
+                    const Real *const row[2] = {p0, p1};
+                    const Real w[2] = {w0, w1};
+                    mv_rows<Real, VPT, kReread, 2>(row, w, opmem, pc, acc, dacc, m, slots, phase, ea,
+                                                   eb);
+                } else if (j < nrows) {
+                    none(eb, nullptr);
+                    one(p0, w0, ea);
+                } else {
+                    none(ea, eb);
+                }
+            }
+            base += two ? 2 * rg.R : rg.R;
+            continue;
+        }
+        int rr = m.team;
+        mbar_wait_or_flag(&full[a], (uint32_t)rg.par, timed_out);
+        rg.next();
+        if (rr >= rows) none(ea, nullptr);
+        if constexpr (kPair) {
+            for (; rr + nt < rows; rr += 2 * nt) {
+                const Real w[2] = {n0, n1};
+                const Real *const row[2] = {buf + (size_t)rr * ld, buf + (size_t)(rr + nt) * ld};
+                n0 = weight(base + rr + 2 * nt);
+                n1 = weight(base + rr + 3 * nt);
+                mv_rows<Real, VPT, kReread, 2>(row, w, opmem, pc, acc, dacc, m, slots, phase,
+                                               rr + 2 * nt < rows ? nullptr : ea, nullptr);
+            }
+        }
+        for (; rr < rows; rr += nt) {
+            const Real w = n0;
+            n0 = n1;
+            n1 = weight(base + rr + 2 * nt);
+            one(buf + (size_t)rr * ld, w, rr + nt < rows ? nullptr : ea);
+        }
+        base += rg.R;
+    }
+}
+
+// The chunk's results: the teams' accumulators added in team order (through red,
+// [nteams][ld], free for the consumers' use) into partial g, and the teams' shares of
+// r^T A r into dpart.  Called by every consumer thread.
+template <typename Real, int VPT>
+__device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const MvTeam &m,
+                                          const Chunk<Real> (&acc)[VPT], const RedAcc<Real> &dacc, Real *red,
+                                          double *dsl)
+{
+    constexpr int E = Chunk<Real>::E;
+    const WS<Real> ws(p);
+    Real *dst = ws.part(s, g, 0);
+    double *dp = p.dpart + ((size_t)s * p.G + g) * kDpart;
+    if (m.nteams == 1) {
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            const int c = m.tl + m.tthreads * v;
+            if (c < m.nch) st_chunk(dst + c * E, acc[v]);
+        }
+        if (m.tl == 0) *dp = dacc.value();
+        return;
+    }
+    const int nthreads = m.tthreads * m.nteams;
+    const int ct = (int)threadIdx.x - 32;
+    const size_t ld = (size_t)m.nch * E;
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        const int c = m.tl + m.tthreads * v;
+        if (c < m.nch) st_chunk(red + (size_t)m.team * ld + c * E, acc[v]);
+    }
+    if (m.tl == 0) dsl[m.team] = dacc.value();
+    bar_named(15, nthreads);
+    // the last warp (it has no more chunks of the sum to add than any other) adds the shares
+    if (ct >= nthreads - 32) {
+        double d = m.lane < m.nteams ? dsl[m.lane] : 0.0;
+#pragma unroll
+        for (int o = 8; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (m.lane == 0) *dp = d;
+    }
+    for (int c = ct; c < m.nch; c += nthreads) {
+        Chunk<Real> sum = ld_chunk(red + c * E);
+        for (int t2 = 1; t2 < m.nteams; ++t2) {
+            const Chunk<Real> o = ld_chunk(red + (size_t)t2 * ld + c * E);
+#pragma unroll
+            for (int e = 0; e < E; ++e) sum.v[e] += o.v[e];
+        }
+        st_chunk(dst + c * E, sum);
+    }
+}
+
+// The product as its own launch (grid (G, Q)).  Warp 0 is the producer: one lane streams
+// the chunk's rows, mv_rows consecutive rows (one contiguous block) per stage, into a ring
+// of mv_stages shared-memory stages with cp.async.bulk, completion counted on the stage's
+// "full" mbarrier.  Each consumer warp arrives on the stage's "empty" mbarrier when done,
+// which lets the producer refill it.
+// MODE (MvMode): how a team walks its rows; set with the geometry.
+template <typename Real, int VPT, int MODE>
+__global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512), 1)
+    k_matvec(Params p)
 {
     constexpr int E = Chunk<Real>::E;
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ double dsl[16];
     const int g = blockIdx.x, s = blockIdx.y;
     if (p.st[s].done) return;
     const WS<Real> ws(p);
@@ -151,111 +467,24 @@ __global__ void __launch_bounds__(WIDE ? 544 : (VPT >= 8 ? 352 : 288), 1) k_matv
                 mbar_wait_or_flag(&full[i % S], (uint32_t)((i / S) & 1), timed_out);
         }
     } else {
-        const int ct = threadIdx.x - 32;
-        const int tthreads = 32 * tw;
-        const int team = ct / tthreads, tl = ct - team * tthreads, wt = tl >> 5;
+        const MvTeam m(tw, nteams, nch);
         const Real *pv = ws.vR(s, 0);
-        const Real *wv = ws.w(s);
-        // the operand r: in registers, except with 16 chunks per thread (the widest FP64
-        // rows), where it is read through L1 for every row (it is the same for all rows)
-        constexpr bool kOpL1 = VPT > 8;
-        constexpr int kOpRegs = kOpL1 ? 1 : VPT;
-        Chunk<Real> acc[VPT], pc[kOpRegs];
+        Chunk<Real> acc[VPT], pc[VPT];
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
+            const int c = m.tl + m.tthreads * v;
             zero(acc[v]);
-            if (!kOpL1) {
-                const int c = tl + tthreads * v;
-                if (c < nch) pc[v] = ldg_chunk(pv + c * E);
-                else zero(pc[v]);
-            }
+            if (VPT <= 8 && c < nch) pc[v] = ldg_chunk(pv + c * E);
+            else zero(pc[v]);
         }
         int phase = 0;
-        for (long long i = 0; i < nst; ++i) {
-            const int st = (int)(i % S);
-            mbar_wait_or_flag(&full[st], (uint32_t)((i / S) & 1), timed_out);
-            const long long row0 = r0 + i * R;
-            const int rows = (int)min((long long)R, r1 - row0);
-            const Real *buf = ring + (size_t)st * R * row_elems;
-            for (int rr = team; rr < rows; rr += nteams) {
-                const Real *row = buf + (size_t)rr * row_elems;
-                // the row's weight, loaded before the dot product so that its latency is
-                // hidden behind the product and the team sum instead of following them
-                const Real wrow = wv[row0 + rr];
-                // narrow teams keep their chunks of the row in registers between the dot
-                // product and the weighted sum (one shared-memory read of the row instead
-                // of two); the 16-warp teams of the widest rows, and the 16 chunks per
-                // thread of the widest FP64 rows, have no registers to spare
-                constexpr bool kReread = WIDE || VPT > 8;
-                constexpr int kHeld = kReread ? 1 : VPT;
-                Chunk<Real> dl[kHeld];
-                Real t = Real(0);
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    const int c = tl + tthreads * v;
-                    Chunk<Real> &x = dl[kReread ? 0 : v];
-                    Chunk<Real> &o = pc[kOpL1 ? 0 : v];
-                    if (c < nch) {
-                        x = ld_chunk(row + c * E);
-                        if (kOpL1) o = ldg_chunk(pv + c * E);
-                    } else {
-                        zero(x);
-                        if (kOpL1) zero(o);
-                    }
-#pragma unroll
-                    for (int e = 0; e < E; ++e) t += x.v[e] * o.v[e];
-                }
-#pragma unroll
-                for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                if (tw > 1) {
-                    Real *sl = slots + (size_t)(team * 2 + phase) * 32;
-                    if (lane == 0) sl[wt] = t;
-                    bar_named(1 + team, tthreads);
-                    t = Real(0);
-                    for (int w2 = 0; w2 < tw; ++w2) t += sl[w2];
-                    phase ^= 1;
-                }
-                const Real coef = wrow * t;
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    const int c = tl + tthreads * v;
-                    if (c < nch) {
-                        if (kReread) dl[0] = ld_chunk(row + c * E);
-                        const Chunk<Real> &x = dl[kReread ? 0 : v];
-#pragma unroll
-                        for (int e = 0; e < E; ++e) acc[v].v[e] += coef * x.v[e];
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[st]);
-        }
-        // team accumulators -> CTA partial (teams summed in team order via the ring)
-        Real *dst = ws.part(s, g, 0);
-        if (nteams == 1) {
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                const int c = tl + tthreads * v;
-                if (c < nch) st_chunk(dst + c * E, acc[v]);
-            }
-        } else {
-            bar_named(15, 32 * nteams * tw);   // every consumer is past its last ring read
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                const int c = tl + tthreads * v;
-                if (c < nch) st_chunk(ring + (size_t)team * row_elems + c * E, acc[v]);
-            }
-            bar_named(15, 32 * nteams * tw);
-            for (int c = ct; c < nch; c += 32 * nteams * tw) {
-                Chunk<Real> sum = ld_chunk(ring + c * E);
-                for (int t2 = 1; t2 < nteams; ++t2) {
-                    const Chunk<Real> o = ld_chunk(ring + (size_t)t2 * row_elems + c * E);
-#pragma unroll
-                    for (int e = 0; e < E; ++e) sum.v[e] += o.v[e];
-                }
-                st_chunk(dst + c * E, sum);
-            }
-        }
+        RedAcc<Real> dacc;
+        dacc.init();
+        MvRing rg{0, 0, S, R};
+        mv_chunk<Real, VPT, (MODE != kMvHold), (VPT <= 8 && (VPT <= 4 || MODE != kMvHold))>(r0, r1, ws.w(s) + r0, pv, pc, acc, dacc, m, ring, full,
+                                               empty, rg, true, slots, phase, timed_out);
+        if (nteams > 1) bar_named(15, m.tthreads * nteams);   // past the last ring read
+        mv_finish<Real, VPT>(p, s, g, m, acc, dacc, ring, dsl);
     }
     if (timed_out) atomicCAS(&p.st[s].status, 0, (int)FBSDE_ERR_TIMEOUT);
 }
