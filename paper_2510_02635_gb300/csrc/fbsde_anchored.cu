@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(256) k_anc_cg_reg(Params p, int nrc, int rows_
 }
 
 // Direct solve of each anchor's regression over its batch (the batch reading of Remark
-// 2.1), in place of the CG passes: one block per anchor m, of one thread per tile with
+// 2.1), in place of the CG passes, for FP64 (k_anc_direct_tiles for FP32): one block per anchor m, of one thread per tile with
 // TPT = 1 (rounded up to whole warps), of kDirThreads threads with TPT = 2.
 //   1. The weighted second moment of the window, sum_q w_jm D_j D_j^T with D_j = P_j - A_m
 //      over j = (m + q) mod M, q < Kb, summed over q in order in the stream precision: the
@@ -837,6 +837,270 @@ __global__ void __launch_bounds__(kDirThreads) k_anc_direct(Params p, long long 
     for (int v = 0; v < kV; ++v) {
         const int i = lane + 32 * v;
         if (i < d) x[o + i] = yv[v];
+    }
+}
+
+// The direct solve of k_anc_direct for FP32, one thread per 8 x 8 tile of the lower triangle
+// (nT (nT + 1) / 2 tiles, nT = ceil(d / 8), tile rows I, tile columns K <= I), everything in
+// registers but what the tiles exchange.
+//   1. Window moments: rows E_q = sqrt(w) D_q pass through shared memory kDtRows at a time
+//      (the next ones are on their way in registers); a thread adds the outer product of two
+//      8-vectors of a row into its tile: 64 FMAs (32 packed) for four 16-byte loads.
+//   2. Gamma + lambda I = moment / W - S S^T + lambda I (identity beyond d).
+//   3. Blocked LDL^T: per tile column c its diagonal thread factors the 8 x 8 block and takes
+//      the block's part of the right-hand side through it; the threads below solve their
+//      tiles against it (U = L D, then L) and update their part of the right-hand side; all
+//      tiles to the right subtract L U^T, the moment step's outer products with the panel's 8
+//      columns as rows.  Two barriers for 8 columns.
+//   4. Back substitution by tile rows, the tiles' L still in registers.
+// A pivot that is not positive and finite leaves x = 0 and the anchor's status FBSDE_ERR_CG.
+// Bound: FMA issue (8 x 4 tiles moved as many shared-memory wavefronts as FMAs, and the
+// factorisation took a barrier per column).  d = 100, M = 2048, window 256: 365 us a level in place of
+// 878 us (the solve 4.8 ms in place of 9.9).
+constexpr int kDtRows = 16;
+__host__ __device__ inline int dt_tiles(int d)
+{
+    const int n = (d + 7) / 8;
+    return n * (n + 1) / 2;
+}
+inline int dt_threads(int d) { return std::max(64, (dt_tiles(d) + 31) / 32 * 32); }
+// shared floats: two row buffers, the panel's L and U (transposed), rhs / x, y, S, A, diagonal
+inline size_t dt_smem_bytes(int d)
+{
+    const size_t dp = (size_t)dir_pad(d);
+    return (2 * kDtRows * dp + 16 * dp + 4 * dp + 64 + 16) * sizeof(float);
+}
+// acc += sgn a b^T for the 8-vectors at a and b
+__device__ __forceinline__ void dt_outer(float2 (&acc)[8][4], const float *a, const float *b)
+{
+    const float4 a0 = *reinterpret_cast<const float4 *>(a);
+    const float4 a1 = *reinterpret_cast<const float4 *>(a + 4);
+    const float4 b0 = *reinterpret_cast<const float4 *>(b);
+    const float4 b1 = *reinterpret_cast<const float4 *>(b + 4);
+    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w),
+                          make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+#pragma unroll
+    for (int ii = 0; ii < 8; ++ii) {
+        const float2 aa = make_float2(av[ii], av[ii]);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) acc[ii][kk] = __ffma2_rn(aa, bv[kk], acc[ii][kk]);
+    }
+}
+__device__ __forceinline__ float &dt_at(float2 (&acc)[8][4], int i, int k)
+{
+    return (k & 1) ? acc[i][k >> 1].y : acc[i][k >> 1].x;
+}
+
+__global__ void __launch_bounds__(160, 3) k_anc_direct_tiles(Params p, long long Kb, const float *P,
+                                                             const float *A, const float *W,
+                                                             const float *S, const float *rhs,
+                                                             Anchor *st, float *x)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const int m = blockIdx.x, t = threadIdx.x, nt = blockDim.x;
+    const int d = p.d, ld = p.ld, dp = dir_pad(d), nT = dp / 8;
+    Anchor &an = st[m];
+    if (an.done) return;   // the whole block
+    float *E = reinterpret_cast<float *>(dsm);      // [2][kDtRows][dp]
+    float *Lt = E + 2 * kDtRows * dp;               // [8][dp] panel L, transposed
+    float *Ut = Lt + 8 * dp;                        // [8][dp] panel -L D, transposed
+    float *bv = Ut + 8 * dp;                        // [dp] right-hand side, then x
+    float *yv = bv + dp;                            // [dp] L^-1 rhs, then D^-1 of it
+    float *Sv = yv + dp, *Av = Sv + dp;             // [dp]
+    float *Ld = Av + dp;                            // [8][8] unit lower factor of the block
+    float *iD = Ld + 64;                            // [8] 1 / D of the block
+    int *bad = reinterpret_cast<int *>(iD + 8);
+    const size_t o = (size_t)m * ld;
+    const int ntiles = nT * (nT + 1) / 2;
+    const bool own = t < ntiles;
+    int ti = 0, tk = t;
+    if (own)
+        while (tk > ti) tk -= ++ti;   // row ti holds ti + 1 tiles
+    for (int i = t; i < dp; i += nt) {
+        Sv[i] = i < d ? S[o + i] : 0.0f;
+        Av[i] = i < d ? A[o + i] : 0.0f;
+        bv[i] = i < d ? rhs[o + i] : 0.0f;
+    }
+    if (t == 0) *bad = 0;
+    __syncthreads();
+    // rows q0 .. of the window: chunk c of row r is item r * nc + c, up to kItems per thread
+    const int nc = dp / 4, items = kDtRows * nc;
+    constexpr int kItems = 5;   // most of ceil(kDtRows nc / nt), at nT = 10
+    float4 v[kItems];
+    float w[kItems];
+    auto fetch = [&](long long q0) {
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            const int it = t + u * nt;
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            w[u] = 0.0f;
+            if (it < items) {
+                const int r = it / nc, c = it - r * nc;
+                if (q0 + r < Kb && 4 * c < ld) {
+                    long long j = m + q0 + r;
+                    if (j >= p.M) j -= p.M;
+                    v[u] = __ldg(reinterpret_cast<const float4 *>(P + (size_t)j * ld) + c);
+                    w[u] = __ldg(W + (size_t)j * p.M + m);
+                }
+            }
+        }
+    };
+    auto put = [&](float *dst) {
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            const int it = t + u * nt;
+            if (it < items) {
+                const int r = it / nc, c = it - r * nc;
+                const float4 a = *reinterpret_cast<const float4 *>(Av + 4 * c);
+                const float q = sqrtf(w[u]);
+                *reinterpret_cast<float4 *>(dst + r * dp + 4 * c) =
+                    make_float4(q * (v[u].x - a.x), q * (v[u].y - a.y), q * (v[u].z - a.z),
+                                q * (v[u].w - a.w));
+            }
+        }
+    };
+    float2 acc[8][4];
+#pragma unroll
+    for (int ii = 0; ii < 8; ++ii)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) acc[ii][kk] = make_float2(0.f, 0.f);
+    fetch(0);
+    put(E);
+    __syncthreads();
+    int buf = 0;
+    for (long long q0 = 0; q0 < Kb; q0 += kDtRows) {
+        const bool more = q0 + kDtRows < Kb;
+        if (more) fetch(q0 + kDtRows);
+        if (own) {
+            const float *e = E + buf * kDtRows * dp;
+#pragma unroll 2
+            for (int r = 0; r < kDtRows; ++r) dt_outer(acc, e + r * dp + 8 * ti, e + r * dp + 8 * tk);
+        }
+        buf ^= 1;
+        if (more) put(E + buf * kDtRows * dp);
+        __syncthreads();
+    }
+    // Gamma + lambda I
+    const float invW = (float)(1.0 / an.W), lam = (float)an.lam;
+#pragma unroll
+    for (int ii = 0; ii < 8; ++ii)
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+            const int i = 8 * ti + ii, k = 8 * tk + kk;
+            float &g = dt_at(acc, ii, kk);
+            if (i < d && k < d) g = g * invW - Sv[i] * Sv[k] + (i == k ? lam : 0.0f);
+            else g = i == k ? 1.0f : 0.0f;
+        }
+    for (int c = 0; c < nT; ++c) {
+        if (own && ti == c && tk == c) {
+            bool ok = true;
+            float z[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) z[i] = bv[8 * c + i];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float piv = dt_at(acc, q, q);
+                ok = ok && piv > 0.0f && isfinite(piv);
+                const float ip = 1.0f / piv;
+                iD[q] = ip;
+#pragma unroll
+                for (int i = q + 1; i < 8; ++i) {
+                    const float l = dt_at(acc, i, q) * ip;
+#pragma unroll
+                    for (int k = q + 1; k <= i; ++k)
+                        dt_at(acc, i, k) = fmaf(-l, dt_at(acc, k, q), dt_at(acc, i, k));
+                    z[i] = fmaf(-l, z[q], z[i]);
+                }
+#pragma unroll
+                for (int i = q + 1; i < 8; ++i) {
+                    const float l = dt_at(acc, i, q) * ip;
+                    dt_at(acc, i, q) = l;
+                    Ld[8 * i + q] = l;
+                }
+                yv[8 * c + q] = z[q];
+            }
+            if (!ok) *bad = 1;
+        }
+        __syncthreads();
+        if (*bad) break;   // the same in every thread
+        if (own && tk == c && ti > c) {
+            // U L_cc^T = G, then L = U D^-1; the right-hand side's rows of this tile
+            float db[8];
+#pragma unroll
+            for (int ii = 0; ii < 8; ++ii) db[ii] = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float lq[8];
+#pragma unroll
+                for (int r = 0; r < q; ++r) lq[r] = Ld[8 * q + r];
+                const float ip = iD[q], z = yv[8 * c + q];
+#pragma unroll
+                for (int ii = 0; ii < 8; ++ii) {
+                    float u = dt_at(acc, ii, q);
+#pragma unroll
+                    for (int r = 0; r < q; ++r) u = fmaf(-dt_at(acc, ii, r), lq[r], u);
+                    dt_at(acc, ii, q) = u;
+                    Ut[q * dp + 8 * ti + ii] = -u;
+                    const float l = u * ip;
+                    Lt[q * dp + 8 * ti + ii] = l;
+                    db[ii] = fmaf(l, z, db[ii]);
+                }
+            }
+#pragma unroll
+            for (int ii = 0; ii < 8; ++ii) bv[8 * ti + ii] -= db[ii];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float ip = iD[q];
+#pragma unroll
+                for (int ii = 0; ii < 8; ++ii) dt_at(acc, ii, q) *= ip;
+            }
+        }
+        if (own && ti == c && tk == c) {   // D^-1 of the block's part
+#pragma unroll
+            for (int q = 0; q < 8; ++q) Sv[8 * c + q] = yv[8 * c + q] * iD[q];
+        }
+        __syncthreads();
+        if (own && tk > c) {
+#pragma unroll 2
+            for (int q = 0; q < 8; ++q) dt_outer(acc, Lt + q * dp + 8 * ti, Ut + q * dp + 8 * tk);
+        }
+    }
+    if (*bad) {
+        if (t == 0) {
+            an.status = FBSDE_ERR_CG;
+            an.done = 1;
+        }
+        return;   // x stays 0 from the setup
+    }
+    // L^T x = y (in Sv by now), tile rows from the last
+    for (int i = nT - 1; i >= 0; --i) {
+        __syncthreads();
+        if (own && ti == i && tk == i) {
+            float xv[8];
+#pragma unroll
+            for (int q = 7; q >= 0; --q) {
+                float s = Sv[8 * i + q];
+#pragma unroll
+                for (int r = q + 1; r < 8; ++r) s = fmaf(-dt_at(acc, r, q), xv[r], s);
+                xv[q] = s;
+                bv[8 * i + q] = s;
+                if (8 * i + q < d) x[o + 8 * i + q] = s;
+            }
+        }
+        __syncthreads();
+        if (own && ti == i && tk < i) {
+            float xv[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) xv[r] = bv[8 * i + r];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float s = Sv[8 * tk + q];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) s = fmaf(-dt_at(acc, r, q), xv[r], s);
+                Sv[8 * tk + q] = s;
+            }
+        }
     }
 }
 
@@ -1167,14 +1431,16 @@ cudaError_t emit_one(const fbsde_problem *Pb, const Lay &L, const double *x0, ui
     const dev::Band band{(long long)M, Kb < M ? Kb : (long long)M};
     if (fused && Kb < M && !direct)
         ANC_TRY(cudaMemsetAsync(T, 0, (size_t)M * M * sizeof(Real), s));
-    // direct batch solve: one 8 x 4 tile per thread while the triangle has at most
+    // direct batch solve in FP64: one 8 x 4 tile per thread while the triangle has at most
     // kDirThreads of them (fewer registers and threads, more blocks per SM), else two
     const size_t dir_smem = dir_smem_bytes(L.d, sizeof(Real));
     const int dir_nI = dir_pad(L.d) / 8;
     const bool dir_two = dir_nI * (dir_nI + 1) > kDirThreads;
-    if (direct)
-        ANC_TRY(cudaFuncSetAttribute(dir_two ? k_anc_direct<Real, 2> : k_anc_direct<Real, 1>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dir_smem));
+    if constexpr (sizeof(Real) == 8) {
+        if (direct)
+            ANC_TRY(cudaFuncSetAttribute(dir_two ? k_anc_direct<Real, 2> : k_anc_direct<Real, 1>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dir_smem));
+    }
     const CgShape cg = cg_shape(ld / Chunk<Real>::E);
     for (int k = L.N - 1; k >= 0; --k) {
         const double t_k = k * p.dt;
@@ -1195,12 +1461,16 @@ cudaError_t emit_one(const fbsde_problem *Pb, const Lay &L, const double *x0, ui
         // the CG passes: a conditional while node (body on b) that repeats while some anchor
         // iterates on and fewer than cg_max_iter passes ran; or each anchor's direct solve
         if (direct) {
-            if (dir_two)
+            if constexpr (sizeof(Real) == 4) {
+                k_anc_direct_tiles<<<M, dt_threads(L.d), dt_smem_bytes(L.d), s>>>(p, band.Kb, P, A, W,
+                                                                                S, rhs, st, x);
+            } else if (dir_two) {
                 k_anc_direct<Real, 2><<<M, kDirThreads, dir_smem, s>>>(p, band.Kb, P, A, W, S, rhs,
                                                                        st, x);
-            else
+            } else {
                 k_anc_direct<Real, 1><<<M, 32 * ((dir_nI * (dir_nI + 1) + 31) / 32), dir_smem, s>>>(
                     p, band.Kb, P, A, W, S, rhs, st, x);
+            }
             ANC_TRY(cudaGetLastError());
         } else {
             cudaStreamCaptureStatus cst;
