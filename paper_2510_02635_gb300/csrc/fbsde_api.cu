@@ -710,28 +710,37 @@ cudaError_t run(Params p, const Layout &L, const double *x0, const double *theta
         FBSDE_TRY(FBSDE_K_PARTICLES, LR::particles(p, L, s));
     }
     if (p.tr_x_N || p.tr_y_N) FBSDE_TRY(FBSDE_K_TRACE, LR::trace_forward(p, L, s));
+    // the regression's set-up: over tiles, or one CTA per query (the three-launch CG)
+    auto set_up = [&](int warm) -> cudaError_t {
+        if (L.cg3) {
+            FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, s));
+            FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, warm, s));
+        } else {
+            ps.newton_level = p.newton_level;
+            FBSDE_TRY(FBSDE_K_REDUCE, LR::level_moments(ps, L, warm, s));
+            FBSDE_TRY(FBSDE_K_FINALIZE, LR::level_rhs(ps, L, s));
+        }
+        return cudaSuccess;
+    };
     if (!L.fused) FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-    FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, s));
     p.newton_level = -1;
-    FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 0, s));
+    if ((e = set_up(0)) != cudaSuccess) return e;
     for (int k = p.N - 1; k >= 0; --k) {
         p.level = k;
         if ((e = cg_loop<Real>(p, L, r)) != cudaSuccess) return e;
-        FBSDE_TRY(FBSDE_K_CG_POST, LR::cg_post(p, L, s));
+        FBSDE_TRY(FBSDE_K_CG_POST, L.cg3 ? LR::cg_post(p, L, s) : LR::level_end(p, L, s));
         if (k >= 1) {
+            ps = p;
+            ps.G = L.Gs;
             if (L.fused) {   // the whole level step in one pass over the rows
-                ps = p;
-                ps.G = L.Gs;
                 FBSDE_TRY(FBSDE_K_STEP, LR::step(ps, L, s));
-                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(ps, L, 3, 3, s));
             } else {
                 FBSDE_TRY(FBSDE_K_UPDATE, LR::update(p, L, s));
                 FBSDE_TRY(FBSDE_K_PARTICLES, LR::particles(p, L, s));
                 FBSDE_TRY(FBSDE_K_MOMENTS, LR::moments(p, L, s));
-                FBSDE_TRY(FBSDE_K_REDUCE, LR::reduce(p, L, 3, 3, s));
             }
             p.newton_level = k;
-            FBSDE_TRY(FBSDE_K_FINALIZE, LR::moments_finalize(p, L, 1, s));
+            if ((e = set_up(1)) != cudaSuccess) return e;
         }
     }
     return cudaSuccess;

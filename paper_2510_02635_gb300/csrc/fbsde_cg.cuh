@@ -209,37 +209,28 @@ template <typename Real> struct CgTileSm {
     double sh[4][2];
 };
 
-// Phase B of one tile of 4 lpr coordinates (lpr = 1, 2, .. 32 lanes a row of partials, so
-// 32 / lpr partials are read by a warp at a time): all NT threads of the block.  c's scalars
-// and the step (c.a, c.ok) are read after the first barrier.  Thread 32 + t, t < 4 lpr, owns
-// coordinate t of the tile: its vector loads are issued first.  The partials are read by
-// warps 1 .. kCgWarps at most, so the order of the sums does not depend on NT.
-template <typename Real, int NT>
-__device__ __forceinline__ void cg_tile(const Params &p, int s, int tile, const CgScal &c,
-                                        CgTileSm<Real> &sm)
+// Warps that read the partial vectors of a tile.
+__device__ __forceinline__ int cg_part_warps(const Params &p)
+{
+    const int per = 32 / p.cg_lpr;
+    return min(kCgWarps, (p.G + per - 1) / per);
+}
+
+// The sums of partial vector `vec` of a tile over the groups of each of the warps 1 ..
+// kCgWarps, into sm.hi and sm.lo (cg_join adds the warps after a barrier).  A lane reads four
+// coordinates of every (kCgWarps 32 / lpr)-th partial.
+template <typename Real>
+__device__ __forceinline__ void cg_partials(const Params &p, int s, int tile, int vec,
+                                            CgTileSm<Real> &sm)
 {
     using Part = CgPart<Real>;
     using Acc = typename Part::Acc;
-    static_assert(NT >= 32 * (kCgWarps + 1), "warps of the partial sums");
     constexpr int kB = 4;   // loads in flight per lane
     const WS<Real> ws(p);
     const int lpr = p.cg_lpr, width = 4 * lpr;
-    const int t = (int)threadIdx.x - 32, lane = threadIdx.x & 31, warp = t >> 5;   // warp 0: -1
-    const int i = tile * width + t;
-    const bool own = t >= 0 && t < width && i < p.ld;
-    const bool first = c.t == 0;
-    double rv = 0.0, pv = 0.0, sv = 0.0, xv = 0.0, Sv = 0.0;
-    if (own) {
-        rv = ws.v64(s, 1)[i];
-        xv = ws.v64(s, 0)[i];
-        Sv = ws.v64(s, 3)[i];
-        if (!first) {
-            pv = ws.v64(s, 2)[i];
-            sv = ws.v64(s, 7)[i];
-        }
-    }
+    const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - 1;
     const int per = 32 / lpr, groups = kCgWarps * per;
-    const int warps = min(kCgWarps, (p.G + per - 1) / per);   // warps with a partial to read
+    const int warps = cg_part_warps(p);
     if (warp >= 0 && warp < warps) {
         // the partial vectors g = group, group + groups, .. of this lane's four coordinates
         const int grp = warp * per + lane / lpr;
@@ -248,7 +239,7 @@ __device__ __forceinline__ void cg_tile(const Params &p, int s, int tile, const 
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[e].init();
         if (e0 < p.ld) {   // ld is a multiple of 4
-            const Real *src = ws.part(s, grp, 0) + e0;
+            const Real *src = ws.part(s, grp, vec) + e0;
             const size_t stride = (size_t)p.part_vecs * p.ld * groups;
             for (int g0 = grp; g0 < p.G; g0 += kB * groups, src += kB * stride) {
                 Quad<Real> q[kB];
@@ -301,24 +292,62 @@ __device__ __forceinline__ void cg_tile(const Params &p, int s, int tile, const 
             }
         }
     }
+}
+
+// Coordinate t's sum over the warps: four interleaved runs (independent additions in flight).
+template <typename Real>
+__device__ __forceinline__ double cg_join(const Params &p, const CgTileSm<Real> &sm, int t)
+{
+    using Part = CgPart<Real>;
+    using Acc = typename Part::Acc;
+    const int warps = cg_part_warps(p);
+    Acc a[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u].init();
+    for (int w = 0; w < warps; w += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (w + u < warps) Part::join(a[u], sm.hi[w + u][t], sm.lo[w + u][t]);
+    Part::join(a[0], a[1].hi(), a[1].lo());
+    Part::join(a[2], a[3].hi(), a[3].lo());
+    Part::join(a[0], a[2].hi(), a[2].lo());
+    return a[0].value();
+}
+
+// Phase B of one tile of 4 lpr coordinates (lpr = 1, 2, .. 32 lanes a row of partials, so
+// 32 / lpr partials are read by a warp at a time): all NT threads of the block.  c's scalars
+// and the step (c.a, c.ok) are read after the first barrier.  Thread 32 + t, t < 4 lpr, owns
+// coordinate t of the tile: its vector loads are issued first.  The partials are read by
+// warps 1 .. kCgWarps at most, so the order of the sums does not depend on NT.
+template <typename Real, int NT>
+__device__ __forceinline__ void cg_tile(const Params &p, int s, int tile, const CgScal &c,
+                                        CgTileSm<Real> &sm)
+{
+    static_assert(NT >= 32 * (kCgWarps + 1), "warps of the partial sums");
+    const WS<Real> ws(p);
+    const int lpr = p.cg_lpr, width = 4 * lpr;
+    const int t = (int)threadIdx.x - 32, lane = threadIdx.x & 31, warp = t >> 5;   // warp 0: -1
+    const int i = tile * width + t;
+    const bool own = t >= 0 && t < width && i < p.ld;
+    const bool first = c.t == 0;
+    double rv = 0.0, pv = 0.0, sv = 0.0, xv = 0.0, Sv = 0.0;
+    if (own) {
+        rv = ws.v64(s, 1)[i];
+        xv = ws.v64(s, 0)[i];
+        Sv = ws.v64(s, 3)[i];
+        if (!first) {
+            pv = ws.v64(s, 2)[i];
+            sv = ws.v64(s, 7)[i];
+        }
+    }
+    cg_partials<Real>(p, s, tile, 0, sm);
     __syncthreads();
     if (t < 0 || t >= max(width, 32)) return;   // whole warps
     double sr = 0.0, rr = 0.0;
     if (!c.ok) {
         rr = -1.0;
     } else if (own) {
-        // the warps' sums: four interleaved runs (independent additions in flight)
-        Acc a[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) a[u].init();
-        for (int w = 0; w < warps; w += 4)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (w + u < warps) Part::join(a[u], sm.hi[w + u][t], sm.lo[w + u][t]);
-        Part::join(a[0], a[1].hi(), a[1].lo());
-        Part::join(a[2], a[3].hi(), a[3].lo());
-        Part::join(a[0], a[2].hi(), a[2].lo());
-        const double wi = fma(a[0].value(), c.invW, fma(-Sv, c.sp, c.lambda * rv));
+        const double wi = fma(cg_join<Real>(p, sm, t), c.invW, fma(-Sv, c.sp, c.lambda * rv));
         const double pi = first ? rv : fma(c.beta, pv, rv);
         const double si = first ? wi : fma(c.beta, sv, wi);
         const double rn = fma(-c.a, si, rv);   // the one operation behind the step

@@ -166,6 +166,10 @@ template <typename Real> struct Launch {
     static bool cg_loop_fits(const Layout &L);   // on the current device
     static cudaError_t cg_loop(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t cg_post(const Params &p, const Layout &L, cudaStream_t s);
+    // the same per level over tiles (fbsde_level.cuh)
+    static cudaError_t level_moments(const Params &p, const Layout &L, int warm, cudaStream_t s);
+    static cudaError_t level_rhs(const Params &p, const Layout &L, cudaStream_t s);
+    static cudaError_t level_end(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t cg_reset(const Params &p, cudaGraphConditionalHandle h, cudaStream_t s);
     static cudaError_t trace_forward(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t normals(uint64_t seed, uint32_t s, uint32_t k, uint32_t j0, int nj, int d,

@@ -3,6 +3,7 @@
 #include "fbsde_adjoint.cuh"
 #include "fbsde_cg.cuh"
 #include "fbsde_cg3.cuh"
+#include "fbsde_level.cuh"
 #include "fbsde_kernels.cuh"
 #include "fbsde_matvec.cuh"
 #include "fbsde_sde.cuh"
@@ -352,6 +353,30 @@ template <typename Real>
 cudaError_t Launch<Real>::cg_reset(const Params &p, cudaGraphConditionalHandle h, cudaStream_t s)
 {
     dev::k_cg_reset<Real><<<1, 32, 0, s>>>(p, h);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t Launch<Real>::level_moments(const Params &p, const Layout &L, int warm, cudaStream_t s)
+{
+    const size_t smem = 3 * sizeof(dev::CgTileSm<Real>);
+    cudaError_t e = set_smem(dev::k_level_moments<Real>, smem);
+    if (e != cudaSuccess) return e;
+    dev::k_level_moments<Real><<<dim3(L.cg_nblk, L.Q), dev::kCgThreads, smem, s>>>(p, warm);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t Launch<Real>::level_rhs(const Params &p, const Layout &L, cudaStream_t s)
+{
+    dev::k_level_rhs<Real><<<dim3(L.cg_nblk, L.Q), dev::kTileThreads, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t Launch<Real>::level_end(const Params &p, const Layout &L, cudaStream_t s)
+{
+    dev::k_level_end<Real><<<dim3(L.cg_nblk, L.Q), dev::kTileThreads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
