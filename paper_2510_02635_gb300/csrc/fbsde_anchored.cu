@@ -59,8 +59,10 @@ template <typename Real, bool TN>
 __global__ void __launch_bounds__(256) k_gemm(int Mr, int Nc, int K, int kc,
                                               const Real *__restrict__ A, int lda,
                                               const Real *__restrict__ B, int ldb,
-                                              Real *__restrict__ C, int ldc, dev::Band band)
+                                              Real *__restrict__ C, int ldc, dev::Band band,
+                                              const int *stop)
 {
+    if (stop && *stop) return;   // behind the last pass of a loop
     constexpr int BM = 64, BN = 64, BK = 16;
     __shared__ Real As[BK][BM + 1];
     __shared__ Real Bs[BK][BN + 1];
@@ -197,23 +199,23 @@ __global__ void k_anc_step(Params p, int k, uint32_t sidx, double a, double b, c
     }
 }
 
-// Row norms |X_j|^2 and, with Y, the rows Y_j P_j.  One block per row.
+// Row norms |X_j|^2 and, with Y, the rows Y_j P_j.  One warp per row.
 template <typename Real>
-__global__ void __launch_bounds__(128) k_anc_rows(Params p, const Real *P, const Real *A,
+__global__ void __launch_bounds__(256) k_anc_rows(Params p, const Real *P, const Real *A,
                                                   const double *Y, double *pn, double *an, Real *YP)
 {
-    __shared__ double sm[32 * 2];
-    const int j = blockIdx.x;
+    const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (j >= p.M) return;
     double acc[2] = {0.0, 0.0};
     const double y = Y[j];
-    for (int i = threadIdx.x; i < p.ld; i += blockDim.x) {
+    for (int i = lane; i < p.ld; i += 32) {
         const Real x = P[(size_t)j * p.ld + i], a = A[(size_t)j * p.ld + i];
         acc[0] += (double)x * x;
         acc[1] += (double)a * a;
         YP[(size_t)j * p.ld + i] = (Real)(y * (double)x);
     }
-    bsum(acc, sm);
-    if (threadIdx.x == 0) {
+    dev::warp_sum(acc);
+    if (lane == 0) {
         pn[j] = acc[0];
         an[j] = acc[1];
     }
@@ -316,8 +318,9 @@ template <typename T, int NV> __device__ __forceinline__ void warp_sums(T (&v)[N
 // on the FP32 path the CG passes then run on the FP32 pipe at half the bytes (the FP64 pipe
 // is a small fraction of it on this part); the scalars of each anchor stay FP64.
 template <typename Real>
-__global__ void __launch_bounds__(32 * kAncWarps) k_anc_setup(Params p, int nrc, int nsplit,
-                                                              const Real *A, const Real *G2,
+__global__ void __launch_bounds__(32 * kAncWarps) k_anc_setup(Params p, int nrc,
+                                                              int rows_per_chunk, dev::Band band,
+                                                              int nsplit, const Real *A, const Real *G2,
                                                               const Real *G3, const double *part,
                                                               Anchor *st, Real *S, Real *rhs,
                                                               Real *x, Real *r, Real *pv)
@@ -328,7 +331,9 @@ __global__ void __launch_bounds__(32 * kAncWarps) k_anc_setup(Params p, int nrc,
     Anchor &a = st[m];
     double w[3] = {0.0, 0.0, 0.0};   // column sums of the weights: lane-strided chunks in
                                      // order, then the warp tree
-    for (int c = lane; c < nrc; c += 32) {
+    for (int c = lane; c < nrc; c += 32) {   // chunks off anchor m's window hold no entry
+        const long long j0 = (long long)c * rows_per_chunk;
+        if (!band.hits(j0, min((long long)p.M, j0 + rows_per_chunk), m, m + 1)) continue;
         const double *o = part + ((size_t)c * p.M + m) * 3;
         w[0] += o[0];
         w[1] += o[1];
@@ -1227,7 +1232,7 @@ bool lay(const fbsde_problem *P, Lay &L)
     L.an = take(M * 8);
     L.cs = take((size_t)L.nrc * M * 3 * 8);
     L.st = take(M * sizeof(Anchor));
-    L.cnt = take(4 * sizeof(int));
+    L.cnt = take(8 * sizeof(int));
     L.total = o;
     return true;
 }
@@ -1273,7 +1278,8 @@ struct TcColumnsEpi {
     const Anchor *st;
     double *part;
     int M;
-    static constexpr bool kColSums = true, kPrefetch = true;
+    static constexpr int kSums = 1;
+    static constexpr bool kPrefetch = true;
     struct Col {
         float ap, inv;
         int skip;
@@ -1298,17 +1304,65 @@ struct TcColumnsEpi {
         }
         return c;
     }
-    __device__ __forceinline__ float put(int, int j, int m, float u, const Col &c, const Pre &pr,
-                                         int rr) const
+    __device__ __forceinline__ dev::TcSums<1> put(int, int j, int m, float u, const Col &c,
+                                                  const Pre &pr, int rr) const
     {
-        if (c.skip) return 0.0f;
+        dev::TcSums<1> s;
+        if (c.skip) return s;
         const float t = pr.w[rr] * (u - c.ap) * c.inv;
         T[(size_t)j * M + m] = t;
-        return t;
+        s.v[0] = t;
+        return s;
     }
-    __device__ __forceinline__ void colsum(int tile, int m, float s) const
+    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<1> &s) const
     {
-        part[((size_t)tile * M + m) * 3] = (double)s;
+        part[((size_t)tile * M + m) * 3] = (double)s.v[0];
+    }
+};
+
+// Epilogue of the distances' product P A^T on the tensor cores: the weights and the column
+// sums of w, w Y and w rho over each 128-row tile, straight from the accumulator
+// (k_anc_columns in mode 0, fused: the product is neither written nor read back; 25 us of a
+// level at d = 100, M = 2048).  Tiles off the band are not visited: the caller keeps W zero
+// there, and the sums' readers skip them.
+struct TcWeightsEpi {
+    const double *pn, *an, *Y;
+    float *W;
+    double *part;
+    int M;
+    long long Kb;
+    float ref, scale;
+    static constexpr int kSums = 3;
+    static constexpr bool kPrefetch = false;
+    struct Col {
+        float am;
+    };
+    struct Pre {};
+    __device__ __forceinline__ void prefetch(int, int, const Col &, Pre &) const {}
+    __device__ __forceinline__ Col column(int m) const { return {m >= 0 ? (float)an[m] : 0.0f}; }
+    __device__ __forceinline__ dev::TcSums<3> put(int, int j, int m, float u, const Col &c,
+                                                  const Pre &, int) const
+    {
+        dev::TcSums<3> s;
+        long long off = (long long)j - m;   // position of particle j in anchor m's window
+        if (off < 0) off += M;
+        float w = 0.0f;
+        if (off < Kb) {
+            const float rho = fmaxf((float)pn[j] + c.am - 2.0f * u, 0.0f);
+            w = expf((rho - ref) * scale);
+            s.v[0] = w;
+            s.v[1] = w * (float)Y[j];
+            s.v[2] = w * rho;
+        }
+        W[(size_t)j * M + m] = w;
+        return s;
+    }
+    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<3> &s) const
+    {
+        double *o = part + ((size_t)tile * M + m) * 3;
+        o[0] = (double)s.v[0];
+        o[1] = (double)s.v[1];
+        o[2] = (double)s.v[2];
     }
 };
 
@@ -1323,7 +1377,8 @@ inline bool tc_layout_ok(bool tn, int K, int kc, const void *A, int lda, const v
 
 template <bool TN, class Epi>
 cudaError_t gemm_tc(int Mr, int Nc, int K, int kc, const float *A, int lda, const float *B,
-                    int ldb, const Epi &epi, int *status, cudaStream_t s, dev::Band band)
+                    int ldb, const Epi &epi, int *status, cudaStream_t s, dev::Band band,
+                    const int *stop = nullptr)
 {
     cudaError_t e = cudaFuncSetAttribute(dev::k_gemm_tc<TN, Epi>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1333,21 +1388,22 @@ cudaError_t gemm_tc(int Mr, int Nc, int K, int kc, const float *A, int lda, cons
                     (K + kc - 1) / kc);
     dev::k_gemm_tc<TN, Epi><<<grid, dev::kTcThreads, dev::kTcSmemBytes, s>>>(Mr, Nc, K, kc, A, lda,
                                                                            B, ldb, epi, status,
-                                                                           band);
+                                                                           band, stop);
     return cudaGetLastError();
 }
 
 template <typename Real, bool TN>
 cudaError_t gemm(int Mr, int Nc, int K, int kc, const Real *A, int lda, const Real *B, int ldb,
-                 Real *C, int ldc, int *status, cudaStream_t s, dev::Band band)
+                 Real *C, int ldc, int *status, cudaStream_t s, dev::Band band,
+                 const int *stop = nullptr)
 {
     if constexpr (sizeof(Real) == 4) {
         if (Mr >= 1024 && tc_layout_ok(TN, K, kc, A, lda, B, ldb))
             return gemm_tc<TN>(Mr, Nc, K, kc, A, lda, B, ldb, dev::TcStore{C, Mr, ldc}, status, s,
-                               band);
+                               band, stop);
     }
     const dim3 grid((Nc + 63) / 64, (Mr + 63) / 64, (K + kc - 1) / kc);
-    k_gemm<Real, TN><<<grid, 256, 0, s>>>(Mr, Nc, K, kc, A, lda, B, ldb, C, ldc, band);
+    k_gemm<Real, TN><<<grid, 256, 0, s>>>(Mr, Nc, K, kc, A, lda, B, ldb, C, ldc, band, stop);
     return cudaGetLastError();
 }
 
@@ -1358,25 +1414,28 @@ cudaError_t gemm(int Mr, int Nc, int K, int kc, const Real *A, int lda, const Re
 
 // Loop control of a level's per-anchor CG, a conditional while node of a CUDA graph.
 // cnt: [0] anchors that iterated on in the last pass (k_anc_cg counts them), [1] device
-// status, [2] passes of the current loop, [3] passes of the whole call.
+// status, [2] passes of the current loop, [3] passes of the whole call, [4] the loop is over.
 __global__ void k_anc_loop_reset(int *cnt, cudaGraphConditionalHandle h)
 {
     if (threadIdx.x != 0) return;
     cnt[0] = 0;
     cnt[2] = 0;
+    cnt[4] = 0;
     cudaGraphSetConditional(h, 1u);
 }
 
 // After a pass: go on while some anchor is still iterating and fewer than max_iter passes
-// ran.
+// ran; else the stop word is set, and a pass behind this one in the body does not count.
 __global__ void k_anc_loop_next(int *cnt, int max_iter, cudaGraphConditionalHandle h)
 {
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0 || cnt[4]) return;
     const int active = cnt[0], passes = cnt[2] + 1;
     cnt[0] = 0;
     cnt[2] = passes;
     cnt[3] += 1;
-    cudaGraphSetConditional(h, (active > 0 && passes < max_iter) ? 1u : 0u);
+    const bool go = active > 0 && passes < max_iter;
+    cnt[4] = go ? 0 : 1;
+    cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
 // Block of the register-resident CG pass for rows of nchk 16-byte chunks: nw warps and C
@@ -1429,8 +1488,11 @@ cudaError_t emit_one(const fbsde_problem *Pb, const Lay &L, const double *x0, ui
     // batch reading: the products cover only the band of entries the windows use (tiles and
     // K-splits off it are skipped); T's entries off the band stay zero for the whole solve
     const dev::Band band{(long long)M, Kb < M ? Kb : (long long)M};
-    if (fused && Kb < M && !direct)
-        ANC_TRY(cudaMemsetAsync(T, 0, (size_t)M * M * sizeof(Real), s));
+    // (and W's, which the fused weight pass does not visit)
+    if (fused && Kb < M) {
+        ANC_TRY(cudaMemsetAsync(W, 0, (size_t)M * M * sizeof(Real), s));
+        if (!direct) ANC_TRY(cudaMemsetAsync(T, 0, (size_t)M * M * sizeof(Real), s));
+    }
     // direct batch solve in FP64: one 8 x 4 tile per thread while the triangle has at most
     // kDirThreads of them (fewer registers and threads, more blocks per SM), else two
     const size_t dir_smem = dir_smem_bytes(L.d, sizeof(Real));
@@ -1447,16 +1509,26 @@ cudaError_t emit_one(const fbsde_problem *Pb, const Lay &L, const double *x0, ui
         const double a = (double)k / (double)(k + 1), bb = p.sigma * std::sqrt(p.dt * a);
         k_anc_step<Real><<<152 * 8, 256, 0, s>>>(p, k, sidx, a, bb, P, A);
         ANC_TRY(cudaGetLastError());
-        k_anc_rows<Real><<<M, 128, 0, s>>>(p, P, A, Y, pn, an, YP);
+        k_anc_rows<Real><<<(M + 7) / 8, 256, 0, s>>>(p, P, A, Y, pn, an, YP);
         ANC_TRY(cudaGetLastError());
-        ANC_TRY((gemm<Real, false>(M, M, ld, ld, P, ld, A, ld, G1, M, cnt + 1, s, band)));   // P A^T
         const double rho_ref = p.sigma * p.sigma * p.d * (t_k + (k + 1) * p.dt);
-        k_anc_columns<Real><<<cgrid, 128, 0, s>>>(p, 0, rho_ref, Kb, G1, pn, an, Y, W, T, st, cs);
-        ANC_TRY(cudaGetLastError());
+        if (fused) {   // the weights straight from the product's epilogue
+            if constexpr (sizeof(Real) == 4)
+                ANC_TRY(gemm_tc<false>(M, M, ld, ld, P, ld, A, ld,
+                                       TcWeightsEpi{pn, an, Y, W, cs, M, Kb, (float)rho_ref,
+                                                    p.uniform ? 0.0f
+                                                              : (float)(-1.0 / (p.h2 * rho_ref))},
+                                       cnt + 1, s, band));
+        } else {
+            ANC_TRY((gemm<Real, false>(M, M, ld, ld, P, ld, A, ld, G1, M, cnt + 1, s, band)));   // P A^T
+            k_anc_columns<Real><<<cgrid, 128, 0, s>>>(p, 0, rho_ref, Kb, G1, pn, an, Y, W, T, st, cs);
+            ANC_TRY(cudaGetLastError());
+        }
         ANC_TRY((gemm<Real, true>(M, ld, M, L.kc, W, M, P, ld, G2, ld, cnt + 1, s, band)));    // W^T P
         ANC_TRY((gemm<Real, true>(M, ld, M, L.kc, W, M, YP, ld, G3, ld, cnt + 1, s, band)));   // W^T (Y P)
-        k_anc_setup<Real><<<awarps, 32 * kAncWarps, 0, s>>>(p, L.nrc, L.nsplit, A, G2, G3, cs, st, S,
-                                                           rhs, x, r, pv);
+        k_anc_setup<Real><<<awarps, 32 * kAncWarps, 0, s>>>(
+            p, fused ? nrc_fused : L.nrc, fused ? dev::kTcBM : kRowChunk, band, L.nsplit, A, G2, G3, cs,
+            st, S, rhs, x, r, pv);
         ANC_TRY(cudaGetLastError());
         // the CG passes: a conditional while node (body on b) that repeats while some anchor
         // iterates on and fewer than cg_max_iter passes ran; or each anchor's direct solve
@@ -1497,45 +1569,50 @@ cudaError_t emit_one(const fbsde_problem *Pb, const Lay &L, const double *x0, ui
             ANC_TRY(cudaStreamBeginCaptureToGraph(b, np.conditional.phGraph_out[0], nullptr, nullptr,
                                                   0, cudaStreamCaptureModeRelaxed));
             cudaError_t eb = cudaSuccess;
-            if (fused) {   // T and its column sums straight from the product's epilogue
-                if constexpr (sizeof(Real) == 4)
-                    eb = gemm_tc<false>(M, M, ld, ld, P, ld, pv, ld, TcColumnsEpi{W, T, st, cs, M},
-                                        cnt + 1, b, band);
-            } else {
-                eb = gemm<Real, false>(M, M, ld, ld, P, ld, pv, ld, G1, M, cnt + 1, b, band);   // U = P V^T
+            // two passes per iteration of the loop (an iteration costs a device-side launch of
+            // its body, about 6 us); the second one ends at once if the first was the last
+            for (int u = 0; u < 2 && eb == cudaSuccess; ++u) {
+                const int *stop = u == 0 ? nullptr : cnt + 4;
+                if (fused) {   // T and its column sums straight from the product's epilogue
+                    if constexpr (sizeof(Real) == 4)
+                        eb = gemm_tc<false>(M, M, ld, ld, P, ld, pv, ld, TcColumnsEpi{W, T, st, cs, M},
+                                            cnt + 1, b, band, stop);
+                } else {
+                    eb = gemm<Real, false>(M, M, ld, ld, P, ld, pv, ld, G1, M, cnt + 1, b, band, stop);   // U = P V^T
+                    if (eb == cudaSuccess) {
+                        k_anc_columns<Real><<<cgrid, 128, 0, b>>>(p, 1, 0.0, Kb, G1, pn, an, Y, W, T, st, cs);
+                        eb = cudaGetLastError();
+                    }
+                }
+                if (eb == cudaSuccess)
+                    eb = gemm<Real, true>(M, ld, M, L.kc, T, M, P, ld, G2, ld, cnt + 1, b, band, stop);   // T^T P
                 if (eb == cudaSuccess) {
-                    k_anc_columns<Real><<<cgrid, 128, 0, b>>>(p, 1, 0.0, Kb, G1, pn, an, Y, W, T, st, cs);
+                    const int nrc_cg = fused ? nrc_fused : L.nrc;
+                    const int rpc = fused ? dev::kTcBM : kRowChunk;
+                    switch (cg.C) {
+                    case 1:
+                        k_anc_cg_reg<Real, 1><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
+                                                                       A, G2, cs, S, st, x, r, pv, cnt);
+                        break;
+                    case 2:
+                        k_anc_cg_reg<Real, 2><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
+                                                                       A, G2, cs, S, st, x, r, pv, cnt);
+                        break;
+                    case 4:
+                        k_anc_cg_reg<Real, 4><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
+                                                                       A, G2, cs, S, st, x, r, pv, cnt);
+                        break;
+                    default:
+                        k_anc_cg<Real><<<awarps, 32 * kAncWarps, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
+                                                                         A, G2, cs, S, st, x, r, pv, q,
+                                                                         cnt);
+                    }
                     eb = cudaGetLastError();
                 }
-            }
-            if (eb == cudaSuccess)
-                eb = gemm<Real, true>(M, ld, M, L.kc, T, M, P, ld, G2, ld, cnt + 1, b, band);   // T^T P
-            if (eb == cudaSuccess) {
-                const int nrc_cg = fused ? nrc_fused : L.nrc;
-                const int rpc = fused ? dev::kTcBM : kRowChunk;
-                switch (cg.C) {
-                case 1:
-                    k_anc_cg_reg<Real, 1><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
-                                                                   A, G2, cs, S, st, x, r, pv, cnt);
-                    break;
-                case 2:
-                    k_anc_cg_reg<Real, 2><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
-                                                                   A, G2, cs, S, st, x, r, pv, cnt);
-                    break;
-                case 4:
-                    k_anc_cg_reg<Real, 4><<<M, 32 * cg.nw, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
-                                                                   A, G2, cs, S, st, x, r, pv, cnt);
-                    break;
-                default:
-                    k_anc_cg<Real><<<awarps, 32 * kAncWarps, 0, b>>>(p, nrc_cg, rpc, band, L.nsplit,
-                                                                     A, G2, cs, S, st, x, r, pv, q,
-                                                                     cnt);
+                if (eb == cudaSuccess) {
+                    k_anc_loop_next<<<1, 32, 0, b>>>(cnt, p.cg_max_iter, h);
+                    eb = cudaGetLastError();
                 }
-                eb = cudaGetLastError();
-            }
-            if (eb == cudaSuccess) {
-                k_anc_loop_next<<<1, 32, 0, b>>>(cnt, p.cg_max_iter, h);
-                eb = cudaGetLastError();
             }
             cudaGraph_t ended = nullptr;
             const cudaError_t ee = cudaStreamEndCapture(b, &ended);
@@ -1559,7 +1636,7 @@ cudaError_t emit_call(const fbsde_problem *P, const Lay &L, int64_t K, bool dire
                       double *grad_u0, char *ws, cudaStream_t s, cudaStream_t b)
 {
     cudaError_t e;
-    ANC_TRY(cudaMemsetAsync(ws + L.cnt, 0, 4 * sizeof(int), s));
+    ANC_TRY(cudaMemsetAsync(ws + L.cnt, 0, 8 * sizeof(int), s));
     for (int q = 0; q < Q; ++q) {
         const double *xq = x0 + (size_t)q * P->d;
         double *gq = grad_u0 ? grad_u0 + (size_t)q * P->d : nullptr;

@@ -205,22 +205,38 @@ struct Band {
     }
 };
 
+// N sums of one output column, added row by row.
+template <int N> struct TcSums {
+    float v[N > 0 ? N : 1];
+    __device__ __forceinline__ TcSums()
+    {
+#pragma unroll
+        for (int i = 0; i < (N > 0 ? N : 1); ++i) v[i] = 0.0f;
+    }
+    __device__ __forceinline__ void add(const TcSums &o)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] += o.v[i];
+    }
+};
+
 // Plain epilogue: C + z Mr ldc gets split z's product.
 struct TcStore {
     float *C;
     int Mr, ldc;
-    static constexpr bool kColSums = false, kPrefetch = false;
+    static constexpr int kSums = 0;
+    static constexpr bool kPrefetch = false;
     struct Col {};
     struct Pre {};
     __device__ __forceinline__ Col column(int) const { return {}; }
     __device__ __forceinline__ void prefetch(int, int, const Col &, Pre &) const {}
-    __device__ __forceinline__ float put(int z, int row, int col, float v, const Col &,
-                                         const Pre &, int) const
+    __device__ __forceinline__ TcSums<0> put(int z, int row, int col, float v, const Col &,
+                                             const Pre &, int) const
     {
         C[((size_t)z * Mr + row) * ldc + col] = v;
-        return 0.0f;
+        return {};
     }
-    __device__ __forceinline__ void colsum(int, int, float) const {}
+    __device__ __forceinline__ void colsum(int, int, const TcSums<0> &) const {}
 };
 
 // Sum_k A(r, k) B(c, k) over k in [z kc, min(K, (z + 1) kc)) for split z = blockIdx.z
@@ -229,9 +245,10 @@ struct TcStore {
 // handed to the epilogue Epi element by element: Epi::column(c) once per output column,
 // Epi::prefetch(r0, c, column state, pre) for the 32 rows r0.. a warp hands out next
 // (issued before the accumulator is read, so its loads overlap that),
-// Epi::put(z, r, c, value, column state, pre, r - r0), whose return values are summed over the rows of
-// the block's 128-row tile (rows in order, 32-row quarters in order) and, with
-// Epi::kColSums, passed to Epi::colsum(row tile, c, sum).
+// Epi::put(z, r, c, value, column state, pre, r - r0), whose Epi::kSums return values are
+// summed over the rows of the block's 128-row tile (rows in order, 32-row quarters in order)
+// and passed to Epi::colsum(row tile, c, sums).  stop (or null): a word that, when not 0, ends
+// the launch at once (a pass behind the last one of a loop).
 // Grid (ceil(Nc / 128), ceil(Mr / 128), splits), kTcThreads threads, kTcSmemBytes of
 // dynamic shared memory.  A wait that times out sets *status = FBSDE_ERR_TIMEOUT (if 0).
 // Band (batch reading): NT products (rows j, columns m) skip tiles that hold no used entry,
@@ -241,8 +258,10 @@ struct TcStore {
 template <bool TN, class Epi>
 __global__ void __launch_bounds__(kTcThreads, 3)
     k_gemm_tc(int Mr, int Nc, int K, int kc, const float *__restrict__ A, int lda,
-              const float *__restrict__ B, int ldb, Epi epi, int *status, Band band)
+              const float *__restrict__ B, int ldb, Epi epi, int *status, Band band,
+              const int *stop = nullptr)
 {
+    if (stop && *stop) return;
     extern __shared__ __align__(1024) uint8_t tsm[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(tsm + kTcStages * kTcStageBytes);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + kTcStages);
@@ -321,7 +340,7 @@ __global__ void __launch_bounds__(kTcThreads, 3)
     // 32 columns at a time, and hands them out row by row through a padded shared-memory
     // transpose (coalesced along the output rows).  The stages are free by now.
     float *scr = reinterpret_cast<float *>(tsm) + warp * (32 * 33);
-    float *csm = reinterpret_cast<float *>(tsm) + 8 * (32 * 33);   // [quarter][column]
+    float *csm = reinterpret_cast<float *>(tsm) + 8 * (32 * 33);   // [sum][quarter][column]
     const int q = warp & 3, h = warp >> 2;
 #pragma unroll 1
     for (int cb = 0; cb < 2; ++cb) {
@@ -340,31 +359,38 @@ __global__ void __launch_bounds__(kTcThreads, 3)
 #pragma unroll
         for (int j = 0; j < 32; ++j) scr[lane * 33 + j] = __uint_as_float(v[j]);
         __syncwarp();
-        float sum = 0.0f;
+        TcSums<Epi::kSums> sum;
         if constexpr (Epi::kPrefetch) {   // pre is indexed by rr: unroll fully
 #pragma unroll
             for (int rr = 0; rr < 32; ++rr) {
                 const int row = r0 + 32 * q + rr;
                 if (row < Mr && cc < Nc)
-                    sum += epi.put(blockIdx.z, row, cc, scr[rr * 33 + lane], cst, pre, rr);
+                    sum.add(epi.put(blockIdx.z, row, cc, scr[rr * 33 + lane], cst, pre, rr));
             }
         } else {
 #pragma unroll 4
             for (int rr = 0; rr < 32; ++rr) {
                 const int row = r0 + 32 * q + rr;
                 if (row < Mr && cc < Nc)
-                    sum += epi.put(blockIdx.z, row, cc, scr[rr * 33 + lane], cst, pre, rr);
+                    sum.add(epi.put(blockIdx.z, row, cc, scr[rr * 33 + lane], cst, pre, rr));
             }
         }
-        if (Epi::kColSums) csm[q * kTcBN + col + lane] = sum;
+#pragma unroll
+        for (int i = 0; i < Epi::kSums; ++i) csm[(4 * i + q) * kTcBN + col + lane] = sum.v[i];
         __syncwarp();
     }
-    if constexpr (Epi::kColSums) {
+    if constexpr (Epi::kSums > 0) {
         __syncthreads();
         const int t = threadIdx.x;
-        if (t < kTcBN && c0 + t < Nc)
-            epi.colsum(blockIdx.y, c0 + t,
-                       ((csm[t] + csm[kTcBN + t]) + csm[2 * kTcBN + t]) + csm[3 * kTcBN + t]);
+        if (t < kTcBN && c0 + t < Nc) {
+            TcSums<Epi::kSums> sum;
+#pragma unroll
+            for (int i = 0; i < Epi::kSums; ++i) {
+                const float *c = csm + 4 * i * kTcBN + t;
+                sum.v[i] = ((c[0] + c[kTcBN]) + c[2 * kTcBN]) + c[3 * kTcBN];
+            }
+            epi.colsum(blockIdx.y, c0 + t, sum);
+        }
     }
     if (timed_out && status) atomicCAS(status, 0, (int)FBSDE_ERR_TIMEOUT);
     tc_fence_before();
