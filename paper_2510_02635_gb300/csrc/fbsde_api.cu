@@ -262,7 +262,9 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
         L.st_vm = L.st_vm1;
         L.st_nslot = 2;
         const size_t ring = (size_t)2 * R * L.ld;
-        const size_t red = L.st_RG > 1 ? (size_t)L.st_RG * 3 * nch * 4 : 0;
+        const bool held = R > 1 && L.st_vm1 <= kStepHeld;
+        const size_t red = held ? (size_t)R * 3 * nch * 4
+                                : (L.st_RG > 1 ? (size_t)L.st_RG * 3 * nch * 4 : 0);
         L.st_region = std::max(ring, red);
         const size_t tail = L.st_vm3 > 5 ? (size_t)3 * (nch - 5 * 480) * 16 : 0;
         L.st_smem = (3 * (size_t)L.ld + L.st_region) * sizeof(float) + 4 * 32 * 16 + 48 + tail;
@@ -275,9 +277,14 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     L.Gs = L.G;
     if (L.fused) {
         const long long gmax_s = std::max<long long>(1, P->M / (4LL * L.st_R));
+        // a cloud too small for that on every SM takes one wave of CTAs with fewer stages
+        // (d = 64, M = 512: 17 CTAs of one stage in place of 4 of four,
+        // 16.6 -> 7.7 us a level)
+        const long long gone = std::max<long long>(gmax_s, (P->M + L.st_R - 1) / L.st_R);
         double best = -1.0;
         for (int W : {4, 3, 2, 1, 5, 6, 7, 8}) {
-            const long long g = std::min<long long>(gmax_s, (152LL * W + Q - 1) / Q);
+            const long long g = std::min<long long>(W == 1 && gmax_s * Q < 152 ? gone : gmax_s,
+                                                    (152LL * W + Q - 1) / Q);
             const double waves = (double)(g * Q) / 152.0;
             const double eff = waves / std::ceil(waves);
             if (eff > best + 1e-9) {

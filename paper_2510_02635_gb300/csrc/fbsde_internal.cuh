@@ -51,6 +51,7 @@ constexpr int kMinRowsPerCta = 32;   // rows of a streaming pass per CTA at leas
                                      // partial vectors for the reduction of small clouds
 constexpr int kRowBlocks = 152 * 8;  // grid of the row-segment kernels (grid-stride)
 constexpr int kStepMaxLd = 10240;    // widest FP32 row of the fused per-level step
+constexpr int kStepHeld = 4;         // chunks per thread its column pass takes from registers
 constexpr int kStepElems = 10240;    // particle-dims per stage of the fused step
 
 struct SolveState {

@@ -23,9 +23,13 @@
 //                    that matters: 64 cycles per dependent FP64 operation on this part),
 //                    the weight, the three moment coefficients; it runs while the
 //                    consumers step the next stage;
-//   P3 (consumers)   each thread owns fixed column chunks and adds the stage's updated rows,
-//                    read back from L2 (they were written one stage earlier), weighted by
-//                    the three coefficients, into register accumulators.
+//   P3 (consumers)   the stage's updated rows, weighted by the three coefficients, are added
+//                    into register accumulators.  With several rows per stage and at most
+//                    kStepHeld chunks per thread, each thread adds the chunks it stepped
+//                    itself, still in registers, and the teams' sums are added at the end.
+//                    Otherwise each thread owns fixed column chunks and reads the rows back
+//                    from L2 (they were written one stage earlier).  (d = 1000, 64
+//                    queries: 860 us a level read back, 823 us held.)
 // P3 of stage i-1 follows P1 of stage i, so P2 is off the consumers' critical path.
 // Hand-offs by mbarriers (b = i mod 2): sums[b] "stage i stepped: row sums written, ring
 // slot free" (every consumer arrives, the service warp waits), coefb[b] "coefficients of
@@ -179,6 +183,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
     // chunks of the column pass held in registers; its sixth chunk (R = 1 with rows wider
     // than 9600 floats) accumulates in shared memory
     constexpr int VMR = VM < 5 ? VM : 5;
+    constexpr bool HELD = !ONE && VM <= kStepHeld;   // P3 from P1's registers
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int g = blockIdx.x, s = blockIdx.y;
     const WS<float> ws(p);
@@ -354,6 +359,11 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
 #pragma unroll
     for (int v = 0; v < VMR; ++v)
         acc[0][v] = acc[1][v] = acc[2][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // HELD: the chunks this thread stepped in the stage before and in this one; chunks past
+    // the row stay 0, rows past the stage are masked by their coefficients
+    float4 prev[HELD ? VM : 1], cur[HELD ? VM : 1];
+#pragma unroll
+    for (int v = 0; v < (HELD ? VM : 1); ++v) prev[v] = cur[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     // fma of one chunk of a row into the three accumulators of chunk v
     auto acc3 = [&](float4 (&a)[3], const float4 cf, const float4 x) {
         const float2 xl = lo2(x), xh = hi2(x);
@@ -408,6 +418,20 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             return;
         }
         mbar_wait_or_flag(&coefb[b], (uint32_t)((i >> 1) & 1), timed_out);
+        if constexpr (HELD) {   // the team's own row, from registers
+            if (team < nrows) {
+                const float4 cf = coef[b * 32 + team];
+#pragma unroll
+                for (int v = 0; v < VMR; ++v) {
+                    float4 a[3] = {acc[0][v], acc[1][v], acc[2][v]};
+                    acc3(a, cf, prev[v]);
+                    acc[0][v] = a[0];
+                    acc[1][v] = a[1];
+                    acc[2][v] = a[2];
+                }
+            }
+            return;
+        }
         if (rg < RG) {
             for (int r = rg; r < nrows; r += RG) {
                 const float4 cf = coef[b * 32 + r];
@@ -471,6 +495,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
                                                            : s1 + ((tx.x + tx.y) + (tx.z + tx.w));
                         }
                         dst[c] = z;
+                        if (HELD) cur[HELD ? v : 0] = z;
                     }
                 }
             }
@@ -506,6 +531,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
                             s2 += (cos_ftz(xa.x) + cos_ftz(xa.y)) + (cos_ftz(xb.x) + cos_ftz(xb.y));
                         }
                         dst[c] = dn;
+                        if (HELD) cur[HELD ? v : 0] = dn;
                     }
                 }
             }
@@ -528,10 +554,39 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
         }
         mbar_arrive(&sums[b]);
         if (i >= 1) p3(i - 1);
+        if (HELD) {
+#pragma unroll
+            for (int v = 0; v < (HELD ? VM : 1); ++v) prev[v] = cur[v];
+        }
     }
     if (nst >= 1) p3(nst - 1);
     if (timed_out) atomicCAS(&st.status, 0, (int)FBSDE_ERR_TIMEOUT);
 
+    if constexpr (HELD) {   // the teams' sums, added in team order
+        bar_named(kStepBarEnd, kStepConsumers);   // every consumer is past its last ring read
+        float4 *red = reinterpret_cast<float4 *>(ring);   // [R][3][nch]
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int v = 0; v < VMR; ++v) {
+                const int c = tl0 + T * v;
+                if (c < nch) red[((size_t)team * 3 + a) * nch + c] = acc[a][v];
+            }
+        bar_named(kStepBarEnd, kStepConsumers);
+        for (int idx = ct; idx < 3 * nch; idx += kStepConsumers) {
+            const int a = idx / nch, c = idx - a * nch;
+            float4 sum = red[(size_t)a * nch + c];
+            for (int r = 1; r < R; ++r) {
+                const float4 o = red[((size_t)r * 3 + a) * nch + c];
+                sum.x += o.x;
+                sum.y += o.y;
+                sum.z += o.z;
+                sum.w += o.w;
+            }
+            reinterpret_cast<float4 *>(ws.part(s, g, a))[c] = sum;
+        }
+        return;
+    }
     // per-CTA partial d-vectors: row groups summed in group order (threads past the RG
     // row groups of tpr threads own no chunk)
     if (RG == 1) {
