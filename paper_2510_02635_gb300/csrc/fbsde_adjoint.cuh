@@ -17,6 +17,7 @@
 // level k (both use the rows Delta_{k+1}).
 #pragma once
 #include "fbsde_kernels.cuh"
+#include "fbsde_level.cuh"
 
 namespace fbsde {
 namespace dev {
@@ -133,65 +134,76 @@ __global__ void __launch_bounds__(kFinThreads) k_adj_warm(Params p)
 // 1/W; weights via p.w), right-hand side alphaxbar - alphabar S.  Start from 0, or with
 // warm = 1 from the guess of k_adj_warm, whose unnormalised product sum_j w_j (D_j . x) D_j
 // is in slot 5: r = rhs - (Gamma_c + lambda I) x.
+// Over the CG's tiles; the query's last tile sets the scalars the CG starts from (d = 1000, one
+// query: 13.4 us with one CTA per query, 6 us here).  Shares (|rhs|^2, |r|^2, S . r) in slot 2.
 template <typename Real>
-__global__ void __launch_bounds__(kFinThreads) k_adj_setup(Params p, int warm)
+__global__ void __launch_bounds__(kTileThreads) k_adj_setup(Params p, int warm)
 {
-    __shared__ double sm[32 * 4];
-    const int s = blockIdx.x, k = p.level;
+    __shared__ double tsm[4][3];
+    __shared__ int flag;
+    const int s = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, k = p.level;
     const WS<Real> ws(p);
     const Tape tp(p);
     SolveState &st = p.st[s];
-    const double *Sk = tp.S(s, k), *ab = tp.av(s, 0);
-    double *x = ws.v64(s, 0), *r = ws.v64(s, 1), *pp = ws.v64(s, 2), *S = ws.v64(s, 3);
-    const double *Gx = ws.v64(s, 5);
-    Real *pR = ws.vR(s, 0);
-    const double abar = st.abar;
     const double *sc = tp.scal(s, k);
-    const double lam = sc[0], invW = sc[1], sx = st.sx;
-    double a[3] = {0.0, 0.0, 0.0};  // |rhs|^2, |r|^2, S.r
-    #pragma unroll 4
-    for (int i = threadIdx.x; i < p.ld; i += blockDim.x) {
-        S[i] = Sk[i];
-        const double rhs = ab[i] - abar * Sk[i];
-        double ri = rhs;
-        if (warm) ri -= Gx[i] * invW - Sk[i] * sx + lam * x[i];
-        else x[i] = 0.0;
-        r[i] = ri;
-        pp[i] = ri;
-        pR[i] = (Real)ri;
-        a[0] += rhs * rhs;
-        a[1] += ri * ri;
-        a[2] += Sk[i] * ri;
+    const double lam = sc[0], invW = sc[1];
+    const int width = 4 * p.cg_lpr, i = tile * width + t;
+    double a[3] = {0.0, 0.0, 0.0};
+    if (t < width && i < p.ld) {
+        const double S = tp.S(s, k)[i], x = warm ? ws.v64(s, 0)[i] : 0.0;
+        const double rhs = tp.av(s, 0)[i] - st.abar * S;
+        double r = rhs;
+        if (warm) r -= ws.v64(s, 5)[i] * invW - S * st.sx + lam * x;
+        else ws.v64(s, 0)[i] = 0.0;
+        ws.v64(s, 3)[i] = S;
+        ws.v64(s, 1)[i] = r;
+        ws.vR(s, 0)[i] = (Real)r;
+        a[0] = rhs * rhs;
+        a[1] = r * r;
+        a[2] = S * r;
     }
-    block_sum(a, sm);
-    if (threadIdx.x == 0) {
+    tile_put(a, tsm, t, ws.v64(s, 2) + 4 * tile);
+    if (!tile_last(p, s, &flag) || t >= 32) return;
+    double v[3];
+    tile_shares(ws.v64(s, 2), p.nblk, v);
+    if (t == 0) {
         st.lambda = lam;
         st.invW = invW;
-        st.rr = a[1];
-        st.rhs2 = a[0];
-        st.sp = a[2];
+        st.rr = v[1];
+        st.rhs2 = v[0];
+        st.sp = v[2];
         st.iters = 0;
-        st.done = (a[1] <= p.cg_tol2 * a[0]) ? 1 : 0;
+        st.done = (v[1] <= p.cg_tol2 * v[0]) ? 1 : 0;
     }
 }
 
-// After the adjoint CG: v in the stream precision for the row pass, S.v.
+// After the adjoint CG: v in the stream precision for the row pass, S.v, and the z quantities
+// of level k + 1 (sum alpha_x, |alpha_x|^2) for its Newton adjoint.
 template <typename Real>
 __global__ void __launch_bounds__(kFinThreads) k_adj_post(Params p)
 {
     __shared__ double sm[32 * 4];
     const int s = blockIdx.x;
     const WS<Real> ws(p);
+    const Tape tp(p);
     const double *x = ws.v64(s, 0), *S = ws.v64(s, 3);
+    const double *ax = p.level + 1 < p.N ? tp.ax(s, p.level + 1) : nullptr;
     Real *xR = ws.vR(s, 1);
-    double a[1] = {0.0};
+    double a[3] = {0.0, 0.0, 0.0};
     #pragma unroll 4
     for (int i = threadIdx.x; i < p.ld; i += blockDim.x) {
         xR[i] = (Real)x[i];
         a[0] += S[i] * x[i];
+        const double z = ax ? ax[i] : 0.0;
+        a[1] += z;
+        a[2] += z * z;
     }
     block_sum(a, sm);
-    if (threadIdx.x == 0) p.st[s].sv = a[0];
+    if (threadIdx.x == 0) {
+        p.st[s].sv = a[0];
+        p.st[s].sumz_l = p.sigma * a[1];
+        p.st[s].zz_l = p.sigma * p.sigma * a[2];
+    }
 }
 
 // Row pass on Delta_{k+1}: per-segment sums of (Delta . v, sum_i cos(x0_i + Delta_i)).
@@ -411,27 +423,33 @@ __global__ void __launch_bounds__(256) k_adj_colsum(Params p, int mode_b, int mo
 //   L < N: alphabar = sum gamma, alphaxbar = sum gamma Delta_L + sigma dt sum gamma df/dz,
 //          x0bar += sum (dt gamma df/dx);
 //   L = N: x0bar += grad g terms, thetabar += d_theta g terms.
-// Also loads the level-L quantities of z for the next particle pass.
+// Blocks of kTileThreads coordinates, each adding the scalar partials itself (one CTA per query
+// took 8.2 us at d = 1000, every thread adding them in turn; 5 us here).
 template <typename Real>
-__global__ void __launch_bounds__(kFinThreads) k_adj_finalize(Params p)
+__global__ void __launch_bounds__(kTileThreads) k_adj_finalize(Params p)
 {
-    __shared__ double sm[32 * 4];
-    const int s = blockIdx.x, L = p.level + 1;
+    __shared__ double sh[2];
+    const int s = blockIdx.y, L = p.level + 1;
     const WS<Real> ws(p);
     const Tape tp(p);
     SolveState &st = p.st[s];
-    double sc[2] = {0.0, 0.0};
-    for (int b = 0; b < p.GP; ++b) {
-        sc[0] += ws.spart(s, b)[0];
-        sc[1] += ws.spart(s, b)[1];
+    if (threadIdx.x < 32) {
+        double v[2];
+        tile_shares(ws.spart(s, 0), p.GP, v);
+        if (threadIdx.x == 0) {
+            sh[0] = v[0];
+            sh[1] = v[1];
+        }
     }
+    __syncthreads();
+    const double sc[2] = {sh[0], sh[1]};
+    const int i = blockIdx.x * kTileThreads + threadIdx.x;
     const double *A = ws.v64(s, 3), *B = ws.v64(s, 4), *C = ws.v64(s, 5);
     const double *theta = p.theta;
     double *ab = tp.av(s, 0), *xb = tp.av(s, 1), *tb = tp.av(s, 2);
     if (L < p.N) {
         const double *axL = tp.ax(s, L);
-        #pragma unroll 4
-        for (int i = threadIdx.x; i < p.ld; i += blockDim.x) {
+        if (i < p.ld) {
             double zb = 0.0;
             if (i < p.d) {
                 switch (p.kind) {
@@ -443,9 +461,9 @@ __global__ void __launch_bounds__(kFinThreads) k_adj_finalize(Params p)
             ab[i] = A[i] + zb;
             xb[i] += B[i];
         }
-        if (threadIdx.x == 0) st.abar = sc[0];
+        if (blockIdx.x == 0 && threadIdx.x == 0) st.abar = sc[0];
     } else {
-        for (int i = threadIdx.x; i < p.d; i += blockDim.x) {
+        if (i < p.d) {
             const double th = theta ? theta[i] : 0.0;
             switch (p.kind) {
             case FBSDE_AC_MANUFACTURED:
@@ -462,30 +480,6 @@ __global__ void __launch_bounds__(kFinThreads) k_adj_finalize(Params p)
                 break;
             }
         }
-    }
-    (void)sm;
-}
-
-// Per query: level-L z quantities (sum alpha_x, |alpha_x|^2) for the next Newton adjoint.
-template <typename Real>
-__global__ void __launch_bounds__(kFinThreads) k_adj_zlevel(Params p)
-{
-    __shared__ double sm[32 * 4];
-    const int s = blockIdx.x, L = p.level + 1;
-    const Tape tp(p);
-    double a[2] = {0.0, 0.0};
-    if (L < p.N) {
-        const double *ax = tp.ax(s, L);
-        #pragma unroll 4
-        for (int i = threadIdx.x; i < p.ld; i += blockDim.x) {
-            a[0] += ax[i];
-            a[1] += ax[i] * ax[i];
-        }
-    }
-    block_sum(a, sm);
-    if (threadIdx.x == 0) {
-        p.st[s].sumz_l = p.sigma * a[0];
-        p.st[s].zz_l = p.sigma * p.sigma * a[1];
     }
 }
 

@@ -865,7 +865,6 @@ cudaError_t run_adjoint(Params p, const Layout &L, const double *x0, const doubl
         if ((e = cg_loop<Real>(p, L, r)) != cudaSuccess) return e;
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_post(p, L, s));
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_rows(p, L, s));
-        FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_zlevel(p, L, s));
         FBSDE_TRY(FBSDE_K_ADJOINT, LR::adj_particles(p, L, s));
         const bool terminal = k + 1 == p.N;
         const int mb = terminal ? mode_b : (p.kind == FBSDE_AC_MANUFACTURED ? 1 : 0);

@@ -181,7 +181,6 @@ template <typename Real> struct Launch {
     static cudaError_t adj_setup(const Params &p, const Layout &L, int warm, cudaStream_t s);
     static cudaError_t adj_post(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t adj_rows(const Params &p, const Layout &L, cudaStream_t s);
-    static cudaError_t adj_zlevel(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t adj_particles(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t adj_colsum(const Params &p, const Layout &L, int mode_b, int mode_c,
                                   cudaStream_t s);

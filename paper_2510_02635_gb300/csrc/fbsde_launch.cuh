@@ -415,7 +415,7 @@ cudaError_t Launch<Real>::adj_warm(const Params &p, const Layout &L, cudaStream_
 template <typename Real>
 cudaError_t Launch<Real>::adj_setup(const Params &p, const Layout &L, int warm, cudaStream_t s)
 {
-    dev::k_adj_setup<Real><<<L.Q, kFinThreads, 0, s>>>(p, warm);
+    dev::k_adj_setup<Real><<<dim3(L.cg_nblk, L.Q), dev::kTileThreads, 0, s>>>(p, warm);
     return cudaGetLastError();
 }
 
@@ -430,13 +430,6 @@ template <typename Real>
 cudaError_t Launch<Real>::adj_rows(const Params &p, const Layout &L, cudaStream_t s)
 {
     FBSDE_SEG_DISPATCH(k_adj_rows, p)
-}
-
-template <typename Real>
-cudaError_t Launch<Real>::adj_zlevel(const Params &p, const Layout &L, cudaStream_t s)
-{
-    dev::k_adj_zlevel<Real><<<L.Q, kFinThreads, 0, s>>>(p);
-    return cudaGetLastError();
 }
 
 template <typename Real>
@@ -466,7 +459,8 @@ cudaError_t Launch<Real>::adj_colsum(const Params &p, const Layout &L, int mode_
 template <typename Real>
 cudaError_t Launch<Real>::adj_finalize(const Params &p, const Layout &L, cudaStream_t s)
 {
-    dev::k_adj_finalize<Real><<<L.Q, kFinThreads, 0, s>>>(p);
+    dev::k_adj_finalize<Real>
+        <<<dim3((L.ld + dev::kTileThreads - 1) / dev::kTileThreads, L.Q), dev::kTileThreads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
