@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(kDirThreads) k_anc_direct(Params p, long long 
 // (nT (nT + 1) / 2 tiles, nT = ceil(d / 8), tile rows I, tile columns K <= I), everything in
 // registers but what the tiles exchange.
 //   1. Window moments: rows E_q = sqrt(w) D_q pass through shared memory kDtRows at a time
-//      (the next ones are on their way in registers); a thread adds the outer product of two
+//      (the other blocks of the SM hide their loads); a thread adds the outer product of two
 //      8-vectors of a row into its tile: 64 FMAs (32 packed) for four 16-byte loads.
 //   2. Gamma + lambda I = moment / W - S S^T + lambda I (identity beyond d).
 //   3. Blocked LDL^T: per tile column c its diagonal thread factors the 8 x 8 block and takes
@@ -860,20 +860,21 @@ __global__ void __launch_bounds__(kDirThreads) k_anc_direct(Params p, long long 
 //   4. Back substitution by tile rows, the tiles' L still in registers.
 // A pivot that is not positive and finite leaves x = 0 and the anchor's status FBSDE_ERR_CG.
 // Bound: FMA issue (8 x 4 tiles moved as many shared-memory wavefronts as FMAs, and the
-// factorisation took a barrier per column).  d = 100, M = 2048, window 256: 365 us a level in place of
-// 878 us (the solve 4.8 ms in place of 9.9).
-constexpr int kDtRows = 16;
+// factorisation took a barrier per column).  d = 100, M = 2048, window 256: 318 us a level in
+// place of 878 us (365 us with the next rows prefetched into registers, whose spills cost more
+// than the loads), the solve 4.2 ms in place of 9.9.
+constexpr int kDtRows = 32;
 __host__ __device__ inline int dt_tiles(int d)
 {
     const int n = (d + 7) / 8;
     return n * (n + 1) / 2;
 }
 inline int dt_threads(int d) { return std::max(64, (dt_tiles(d) + 31) / 32 * 32); }
-// shared floats: two row buffers, the panel's L and U (transposed), rhs / x, y, S, A, diagonal
+// shared floats: rows, the panel's L and U (transposed), rhs / x, y, S, A, diagonal
 inline size_t dt_smem_bytes(int d)
 {
     const size_t dp = (size_t)dir_pad(d);
-    return (2 * kDtRows * dp + 16 * dp + 4 * dp + 64 + 16) * sizeof(float);
+    return (kDtRows * dp + 16 * dp + 4 * dp + 64 + 16) * sizeof(float);
 }
 // acc += sgn a b^T for the 8-vectors at a and b
 __device__ __forceinline__ void dt_outer(float2 (&acc)[8][4], const float *a, const float *b)
@@ -907,8 +908,8 @@ __global__ void __launch_bounds__(160, 3) k_anc_direct_tiles(Params p, long long
     const int d = p.d, ld = p.ld, dp = dir_pad(d), nT = dp / 8;
     Anchor &an = st[m];
     if (an.done) return;   // the whole block
-    float *E = reinterpret_cast<float *>(dsm);      // [2][kDtRows][dp]
-    float *Lt = E + 2 * kDtRows * dp;               // [8][dp] panel L, transposed
+    float *E = reinterpret_cast<float *>(dsm);      // [kDtRows][dp]
+    float *Lt = E + kDtRows * dp;                   // [8][dp] panel L, transposed
     float *Ut = Lt + 8 * dp;                        // [8][dp] panel -L D, transposed
     float *bv = Ut + 8 * dp;                        // [dp] right-hand side, then x
     float *yv = bv + dp;                            // [dp] L^-1 rhs, then D^-1 of it
@@ -929,61 +930,48 @@ __global__ void __launch_bounds__(160, 3) k_anc_direct_tiles(Params p, long long
     }
     if (t == 0) *bad = 0;
     __syncthreads();
-    // rows q0 .. of the window: chunk c of row r is item r * nc + c, up to kItems per thread
+    // rows q0 .. of the window: chunk c of row r is item r * nc + c
     const int nc = dp / 4, items = kDtRows * nc;
-    constexpr int kItems = 5;   // most of ceil(kDtRows nc / nt), at nT = 10
-    float4 v[kItems];
-    float w[kItems];
-    auto fetch = [&](long long q0) {
+    float2 acc[8][4];
 #pragma unroll
-        for (int u = 0; u < kItems; ++u) {
-            const int it = t + u * nt;
-            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            w[u] = 0.0f;
-            if (it < items) {
-                const int r = it / nc, c = it - r * nc;
-                if (q0 + r < Kb && 4 * c < ld) {
+    for (int ii = 0; ii < 8; ++ii)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) acc[ii][kk] = make_float2(0.f, 0.f);
+    for (long long q0 = 0; q0 < Kb; q0 += kDtRows) {
+        constexpr int kU = 3;   // items in flight per thread
+        for (int it0 = t; it0 < items; it0 += kU * nt) {
+            float4 v[kU];
+            float w[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int it = it0 + u * nt, r = it / nc, c = it - r * nc;
+                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                w[u] = 0.0f;
+                if (it < items && q0 + r < Kb && 4 * c < ld) {
                     long long j = m + q0 + r;
                     if (j >= p.M) j -= p.M;
                     v[u] = __ldg(reinterpret_cast<const float4 *>(P + (size_t)j * ld) + c);
                     w[u] = __ldg(W + (size_t)j * p.M + m);
                 }
             }
-        }
-    };
-    auto put = [&](float *dst) {
 #pragma unroll
-        for (int u = 0; u < kItems; ++u) {
-            const int it = t + u * nt;
-            if (it < items) {
-                const int r = it / nc, c = it - r * nc;
-                const float4 a = *reinterpret_cast<const float4 *>(Av + 4 * c);
-                const float q = sqrtf(w[u]);
-                *reinterpret_cast<float4 *>(dst + r * dp + 4 * c) =
-                    make_float4(q * (v[u].x - a.x), q * (v[u].y - a.y), q * (v[u].z - a.z),
-                                q * (v[u].w - a.w));
+            for (int u = 0; u < kU; ++u) {
+                const int it = it0 + u * nt, r = it / nc, c = it - r * nc;
+                if (it < items) {
+                    const float4 a = *reinterpret_cast<const float4 *>(Av + 4 * c);
+                    const float q = sqrtf(w[u]);
+                    *reinterpret_cast<float4 *>(E + r * dp + 4 * c) =
+                        make_float4(q * (v[u].x - a.x), q * (v[u].y - a.y), q * (v[u].z - a.z),
+                                    q * (v[u].w - a.w));
+                }
             }
         }
-    };
-    float2 acc[8][4];
-#pragma unroll
-    for (int ii = 0; ii < 8; ++ii)
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) acc[ii][kk] = make_float2(0.f, 0.f);
-    fetch(0);
-    put(E);
-    __syncthreads();
-    int buf = 0;
-    for (long long q0 = 0; q0 < Kb; q0 += kDtRows) {
-        const bool more = q0 + kDtRows < Kb;
-        if (more) fetch(q0 + kDtRows);
+        __syncthreads();
         if (own) {
-            const float *e = E + buf * kDtRows * dp;
+            const int n = (int)min((long long)kDtRows, Kb - q0);
 #pragma unroll 2
-            for (int r = 0; r < kDtRows; ++r) dt_outer(acc, e + r * dp + 8 * ti, e + r * dp + 8 * tk);
+            for (int r = 0; r < n; ++r) dt_outer(acc, E + r * dp + 8 * ti, E + r * dp + 8 * tk);
         }
-        buf ^= 1;
-        if (more) put(E + buf * kDtRows * dp);
         __syncthreads();
     }
     // Gamma + lambda I
