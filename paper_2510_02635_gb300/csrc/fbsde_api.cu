@@ -241,35 +241,46 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
                                             (long long)kRowBlocks);
     // per-particle kernel: 256 particles per block
     L.GP = (int)((P->M + 255) / 256);
-    // fused per-level step (FP32 rows up to kStepMaxLd floats): R rows per stage, the
-    // largest of {1, 3, 5, 15, 30} with R ld <= kStepElems (at most 30: one service-warp lane
-    // per row), T = 480 / R threads per row in the row pass (whole warps, or half-warps at
-    // R = 30), VM = ceil(nch / T) chunks per thread; column pass in row groups of
-    // tpr = min(480, nch) threads; a two-slot ring of stages in shared memory
+    // fused per-level step (FP32 rows up to kStepMaxLd floats): R rows per stage, a service
+    // warp's lane each, and T threads per row (whole warps or half-warps) with
+    // VM = ceil(nch / T) <= 5 chunks each.  Among the T that allow three rows or more, the
+    // one with the most rows per VM + 1 steps of a warp (its chunks, and about one chunk's
+    // time for the sums and hand-offs): d = 1000: 9 rows of 64 threads, 620 us a level (64 queries of 4096), five
+    // rows of 96, 699 us; d = 2503: 4 rows of 128, 73 us (8192 rows), 3 of 160, 78 us.
+    // At most 30 rows (d = 64, 512 rows, 6 levels: 955 us a solve, 990 us with 32).
+    // Otherwise one row of 480 threads.  The column pass lags two stages where the ring
+    // holds five (it frees a slot lag + 1 stages after its row pass, and a slot is requested
+    // at least one stage ahead), else one.
     L.sde = is_sde(P) ? 1 : 0;
     L.fused = !L.sde && P->precision == FBSDE_FP32 && L.ld <= kStepMaxLd;
     if (L.fused) {
-        constexpr int kRows[5] = {1, 3, 5, 15, 30};
-        int R = 1;
-        for (int r : kRows)
-            if ((size_t)r * L.ld <= (size_t)kStepElems) R = r;
-        L.st_R = R;
-        L.st_T = 480 / R;
-        L.st_vm1 = (nch + L.st_T - 1) / L.st_T;
-        L.st_tpr = std::min(480, nch);
-        L.st_RG = 480 / L.st_tpr;
-        L.st_vm3 = (nch + L.st_tpr - 1) / L.st_tpr;
-        L.st_vm = L.st_vm1;
-        L.st_nslot = 2;
-        const size_t ring = (size_t)2 * R * L.ld;
-        const bool held = R > 1 && L.st_vm1 <= kStepHeld;
-        const size_t red = held ? (size_t)R * 3 * nch * 4
-                                : (L.st_RG > 1 ? (size_t)L.st_RG * 3 * nch * 4 : 0);
-        L.st_region = std::max(ring, red);
-        const size_t tail = L.st_vm3 > 5 ? (size_t)3 * (nch - 5 * 480) * 16 : 0;
-        L.st_smem = (3 * (size_t)L.ld + L.st_region) * sizeof(float) + 4 * 32 * 16 + 48 + tail;
-        if (L.st_vm > 6 || L.st_vm3 > L.st_vm || (L.st_vm3 > 5 && R != 1) ||
-            L.st_smem > 227 * 1024)
+        L.st_R = 1;
+        L.st_T = 480;
+        double best_rate = 0.0;
+        for (int T : {16, 32, 64, 96, 128, 160, 192, 288}) {
+            const int vm = (nch + T - 1) / T;
+            long long R = std::min<long long>({kStepMaxConsumers / T, kStepElems / L.ld, 30});
+            if (T < 32) R &= ~1LL;   // whole warps
+            const double rate = (double)R / (vm + 1.0);
+            if (vm <= 5 && R > 2 && rate > best_rate) {
+                best_rate = rate;
+                L.st_R = (int)R;
+                L.st_T = T;
+            }
+        }
+        const int R = L.st_R;
+        L.st_vm = (nch + L.st_T - 1) / L.st_T;
+        // the teams' sums [R][3][nch] of 16 bytes lie over the ring at the end
+        const size_t red = R > 1 ? (size_t)R * 3 * nch * 4 : 0;
+        const size_t tail = R == 1 && nch > 5 * 480 ? (size_t)3 * (nch - 5 * 480) * 16 : 0;
+        for (L.st_nslot = R > 1 ? kStepSlots : 2;; --L.st_nslot) {
+            L.st_region = std::max((size_t)L.st_nslot * R * L.ld, red);
+            L.st_smem = (3 * (size_t)L.ld + L.st_region) * sizeof(float) + 8 * 32 * 16 +
+                        (kStepSlots + 12) * 8 + tail;
+            if (L.st_nslot <= 2 || L.st_smem <= 227 * 1024) break;
+        }
+        L.st_lag = L.st_nslot >= 5 ? 2 : 1;
+        if (L.st_vm > 6 || (R > 1 && L.st_nslot < 3) || L.st_smem > 227 * 1024)
             return FBSDE_ERR_ARG;
     }
     // CTAs per query of the fused step (one CTA per SM): whole waves of 152 CTAs where
@@ -363,10 +374,7 @@ Params make_params(const fbsde_problem *P, const Layout &L, void *ws, uint64_t s
     p.nsp = L.fused ? L.Gs : L.GP;
     p.st_R = L.st_R;
     p.st_T = L.st_T;
-    p.st_vm1 = L.st_vm1;
-    p.st_tpr = L.st_tpr;
-    p.st_RG = L.st_RG;
-    p.st_vm3 = L.st_vm3;
+    p.st_lag = L.st_lag;
     p.st_nslot = L.st_nslot;
     p.st_region = (long long)L.st_region;
     p.mv_rows = L.mv_rows;

@@ -51,8 +51,9 @@ constexpr int kMinRowsPerCta = 32;   // rows of a streaming pass per CTA at leas
                                      // partial vectors for the reduction of small clouds
 constexpr int kRowBlocks = 152 * 8;  // grid of the row-segment kernels (grid-stride)
 constexpr int kStepMaxLd = 10240;    // widest FP32 row of the fused per-level step
-constexpr int kStepHeld = 4;         // chunks per thread its column pass takes from registers
 constexpr int kStepElems = 10240;    // particle-dims per stage of the fused step
+constexpr int kStepMaxConsumers = 576;   // most consumer threads of the fused step
+constexpr int kStepSlots = 8;        // most ring slots (stages) of the fused step
 
 struct SolveState {
     double c, alpha, lambda, invW, rr, rhs2, sp, yref, sumz, zz, phi0, gx0;
@@ -81,8 +82,8 @@ struct Layout {
     int cg3, c3_tw, c3_vpt, c3_teams, c3_rows, c3_stages;
     size_t c3_smem;
     // fused per-level step (FP32 rows of at most kStepMaxLd floats): rows per stage, threads
-    // per row, chunks per thread in the row pass, column-pass row groups, shared memory
-    int fused, st_R, st_T, st_vm1, st_tpr, st_RG, st_vm3, st_vm, st_nslot, GS, Gs;
+    // per row, chunks per thread, ring slots, lag of the column pass in stages
+    int fused, st_R, st_T, st_vm, st_nslot, st_lag, GS, Gs;
     // forward SDE with drift / state-dependent diffusion: checkpoint interval s, checkpoint
     // slabs, slabs in all (checkpoints, then one segment), stored rows and anchor offsets
     int sde, sde_s, sde_ncp, sde_slots;
@@ -103,7 +104,7 @@ struct Params {
     long long M;
     double sigma, T, dt, sdt, A, c0, c1, c2, c3, h2, ridge_rel, cg_tol2, newton_tol;
     double wa, wb;  // path step of the row kernels: Delta <- wa Delta + wb xi (set per launch)
-    int st_R, st_T, st_vm1, st_tpr, st_RG, st_vm3, st_nslot, nsp;  // fused step geometry;
+    int st_R, st_T, st_nslot, st_lag, nsp;  // fused step geometry;
                                                                     // nsp = spart blocks of a level
     long long st_region;  // floats of the fused step's row-slot region
     uint32_t rk0[10], rk1[10];  // Philox4x32-10 round keys of (key0, key1)

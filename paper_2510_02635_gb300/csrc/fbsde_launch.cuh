@@ -144,7 +144,8 @@ static cudaError_t launch_step(const Params &q, const Layout &L, cudaStream_t s)
 {
     cudaError_t e = set_smem(dev::k_step<VM, COSF, TERM, ONE>, L.st_smem);
     if (e != cudaSuccess) return e;
-    dev::k_step<VM, COSF, TERM, ONE><<<dim3(q.G, L.Q), dev::kStepThreads, L.st_smem, s>>>(q);
+    const int threads = ONE ? dev::step_threads(true) : L.st_R * L.st_T + 64;
+    dev::k_step<VM, COSF, TERM, ONE><<<dim3(q.G, L.Q), threads, L.st_smem, s>>>(q);
     return cudaGetLastError();
 }
 
@@ -175,17 +176,25 @@ cudaError_t Launch<Real>::step(const Params &p, const Layout &L, cudaStream_t s)
         }
         const bool term = p.level == p.N;
         const bool cosf = !term && p.kind == FBSDE_AC_MANUFACTURED;
-#define FBSDE_STEP_CASE(VM)                                                              \
+#define FBSDE_STEP_CASE(VM, ONE)                                                         \
     case VM:                                                                             \
-        return L.st_R == 1 ? launch_step_kind<VM, true>(q, L, term, cosf, s)             \
-                           : launch_step_kind<VM, false>(q, L, term, cosf, s);
-        switch (L.st_vm) {
-            FBSDE_STEP_CASE(1)
-            FBSDE_STEP_CASE(2)
-            FBSDE_STEP_CASE(3)
-            FBSDE_STEP_CASE(4)
-            FBSDE_STEP_CASE(5)
-            FBSDE_STEP_CASE(6)
+        return launch_step_kind<VM, ONE>(q, L, term, cosf, s);
+        if (L.st_R == 1) {   // rows of 3416 floats and more
+            switch (L.st_vm) {
+                FBSDE_STEP_CASE(2, true)
+                FBSDE_STEP_CASE(3, true)
+                FBSDE_STEP_CASE(4, true)
+                FBSDE_STEP_CASE(5, true)
+                FBSDE_STEP_CASE(6, true)
+            }
+        } else {
+            switch (L.st_vm) {
+                FBSDE_STEP_CASE(1, false)
+                FBSDE_STEP_CASE(2, false)
+                FBSDE_STEP_CASE(3, false)
+                FBSDE_STEP_CASE(4, false)
+                FBSDE_STEP_CASE(5, false)
+            }
         }
 #undef FBSDE_STEP_CASE
         return cudaErrorInvalidValue;

@@ -8,44 +8,58 @@
 // (k = N) runs the same kernel without the read: the forward sweep's end point, g and the
 // first regression's moments.  Included after fbsde_kernels.cuh.
 //
-// Block: kStepWarps consumer warps + one service warp (16 warps: 128 registers a thread).
-// The CTA owns the contiguous rows [r0, r1) of one query, taken in stages of R rows
-// (R in {1, 3, 5, 15, 30}, R * ld <= kStepElems floats where possible):
-//   load (service warp, one lane)  the rows Delta_{k+1} of stage i + 2 are copied into a
-//                    two-slot shared-memory ring by one bulk copy (cp.async.bulk, completion
-//                    on the slot's mbarrier) as soon as the consumers are done with stage i;
-//   P1 (consumers)   team of T = 480 / R threads per row, VM chunks of 16 bytes each per
-//                    thread: the chunks are read from the ring, stepped and written back to
-//                    HBM; the four row sums (alpha_x . D, |D|^2, sum cos(x0 + D), g . D) go
-//                    to shared memory per warp (or half-warp);
+// Block: consumer warps and service warps.  The CTA owns the contiguous rows [r0, r1) of one
+// query, taken in stages of R rows with a team of T threads per row:
+//   rows above about 3400 floats  R = 1, T = 480 (15 consumer warps and one service warp,
+//                    128 registers a thread), a ring of two stages;
+//   narrower rows    R >= 3, R T <= 576 (up to 18 consumer warps and two service warps, 96
+//                    registers), a ring of 3 to 8 stages.
+//   load (a service warp, one lane)  the rows Delta_{k+1} of a stage are copied into the
+//                    shared-memory ring by one bulk copy (cp.async.bulk, completion on the
+//                    slot's mbarrier) as soon as the consumers are done with the slot;
+//   P1 (consumers)   VM chunks of 16 bytes per thread: read from the ring, stepped, written
+//                    back to HBM and, with several rows, to the ring; the four row sums
+//                    (alpha_x . D, |D|^2, sum cos(x0 + D), g . D) go to shared memory per
+//                    warp (or half-warp);
 //   P2 (service warp) lane r handles row r of the stage: FP32 Newton, then FP64 Newton
 //                    iterations that decide Y_k (the FP64 dependency chain is the latency
 //                    that matters: 64 cycles per dependent FP64 operation on this part),
 //                    the weight, the three moment coefficients; it runs while the
-//                    consumers step the next stage;
+//                    consumers step the next stages;
 //   P3 (consumers)   the stage's updated rows, weighted by the three coefficients, are added
-//                    into register accumulators.  With several rows per stage and at most
-//                    kStepHeld chunks per thread, each thread adds the chunks it stepped
-//                    itself, still in registers, and the teams' sums are added at the end.
-//                    Otherwise each thread owns fixed column chunks and reads the rows back
-//                    from L2 (they were written one stage earlier).  (d = 1000, 64
-//                    queries: 860 us a level read back, 823 us held.)
-// P3 of stage i-1 follows P1 of stage i, so P2 is off the consumers' critical path.
-// Hand-offs by mbarriers (b = i mod 2): sums[b] "stage i stepped: row sums written, ring
-// slot free" (every consumer arrives, the service warp waits), coefb[b] "coefficients of
-// stage i ready" (the service warp arrives, each consumer waits on its own), so the
-// consumer warps never wait for one another and a fast warp may run a stage ahead.  Outputs: the updated rows, Y_k, the weights,
-// per-CTA partial d-vectors (reduced by k_reduce_partials) and per-CTA scalar sums (spart).
+//                    into register accumulators.  One row per stage: read back from L2 (it
+//                    was written one stage earlier).  Several: each thread adds the chunks it
+//                    stepped itself, from the ring, and the teams' sums are added at the end.
+// P3 of stage i - lag follows P1 of stage i, so P2 is off the consumers' critical path (lag 1
+// or 2).  P2 takes about 4800 cycles a stage whatever its rows, and one warp doing it stage
+// after stage bounded the kernel for narrow rows: d = 1000, 64 queries of 4096 particles,
+// five rows a stage, 823 us a level with one service warp (596 us with its Newton iterations
+// left out), 699 us with two of them and a lag of two stages, 620 us with nine rows and 18
+// consumer warps (663 us with 15).  Against 4.2 GB read and written that is 3.4 TB/s; the
+// issue of the normals' arithmetic (43 instructions per particle-dim) bounds it now.
+// Hand-offs by mbarriers: sums[b] "stage i stepped: row sums written" (every consumer arrives,
+// the service warp waits), coefb[b] "coefficients of stage i ready" (the service warp arrives,
+// each consumer waits on its own), so the consumer warps never wait for one another and a fast
+// warp may run ahead by the lag.  Outputs: the updated rows, Y_k, the weights, per-CTA partial
+// d-vectors (reduced by k_reduce_partials or the level kernels) and per-CTA scalar sums (spart).
 #pragma once
 #include "fbsde_matvec.cuh"   // mbarrier and bulk-copy helpers
 
 namespace fbsde {
 namespace dev {
 
-constexpr int kStepWarps = 15;   // + the scalar warp: 16 warps, four per SM sub-partition
-constexpr int kStepConsumers = 32 * kStepWarps;
-constexpr int kStepThreads = kStepConsumers + 32;
+constexpr int kStepConsumers = 480;   // with one row per stage
+// most threads of a block: 15 consumer warps and one service warp with one row per stage,
+// up to 18 and two with several
+constexpr int step_threads(bool one) { return one ? kStepConsumers + 32 : kStepMaxConsumers + 64; }
 constexpr int kStepBarEnd = 5;   // named barrier of the consumers' final reduction
+constexpr int kStepBarSum = 6;   // of the two service warps' scalar sums
+
+// Orders this thread's accesses of shared memory before the bulk copies issued after it.
+__device__ __forceinline__ void fence_async_smem()
+{
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 
 // Philox words of one 16-byte chunk -> the four scaled normals scale * xi (Box-Muller
 // pairs (0,1), (2,3)); bit-identical to normal_chunk for scale = 1.
@@ -171,19 +185,19 @@ __device__ __forceinline__ double newton_fp32_fp64(const Params &p, double E, fl
     return y;
 }
 
-// Geometry of the fused step (host-computed, in Params): R rows per stage, T = 480 / R
-// threads per row in P1 with VM chunks each (VM = ceil(nch / T), the template argument);
-// P3 row groups of tpr threads (RG of them), vm3 <= VM chunks per thread.  ONE: the
-// one-row stage (R = 1, T = tpr = 480, rows wider than
-// 3413 floats) with its strides known at compile time; its chunks v < VM - 1 always lie
-// inside the row.
+// Geometry of the fused step (host-computed, in Params): R rows per stage, T threads per
+// row with VM chunks each (VM = ceil(nch / T), the template argument), NS ring
+// slots, a lag of st_lag stages between the row pass and the column pass.  ONE: the one-row
+// stage (R = 1, T = 480, NS = 2, lag 1) with its strides known
+// at compile time; its chunks v < VM - 1 always lie inside the row.
 template <int VM, bool COSF, bool TERM, bool ONE>
-__global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
+__global__ void __launch_bounds__(step_threads(ONE), 1) k_step(Params p)
 {
-    // chunks of the column pass held in registers; its sixth chunk (R = 1 with rows wider
-    // than 9600 floats) accumulates in shared memory
-    constexpr int VMR = VM < 5 ? VM : 5;
-    constexpr bool HELD = !ONE && VM <= kStepHeld;   // P3 from P1's registers
+    // one row per stage: its sixth chunk (rows wider than 9600 floats) accumulates in
+    // shared memory
+    constexpr int VMR = ONE && VM > 5 ? 5 : VM;
+    constexpr int kBuf = ONE ? 2 : 4;       // buffers of row sums and coefficients
+    constexpr int kService = ONE ? 1 : 2;   // service warps, stage i to warp i mod kService
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int g = blockIdx.x, s = blockIdx.y;
     const WS<float> ws(p);
@@ -191,26 +205,29 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
     constexpr bool terminal = TERM;
     const int ld = p.ld, nch = ld >> 2, d = p.d;
     const int R = ONE ? 1 : p.st_R, T = ONE ? kStepConsumers : p.st_T;
+    const int nc = ONE ? kStepConsumers : R * T;   // consumer threads
     float *vx = reinterpret_cast<float *>(smem_raw);   // alpha_x (terminal: unused)
     float *vg = vx + ld;                                // g (terminal: theta)
     float *vx0 = vg + ld;                               // x0
-    float *ring = vx0 + ld;                             // [2][R][ld] rows Delta_{k+1}
+    float *ring = vx0 + ld;                             // [NS][R][ld] rows Delta_{k+1}
+    const int NS = ONE ? 2 : p.st_nslot, LAG = ONE ? 1 : p.st_lag;
     const size_t slot_floats = (size_t)R * ld;
-    float4 *wsum = reinterpret_cast<float4 *>(ring + p.st_region);    // [2][32]
-    float4 *coef = wsum + 64;                                            // [2][32]
-    // mbarriers: full[2] ring slot loaded (bulk-copy bytes), sums[2] row sums of a stage
-    // written by every consumer thread, coefb[2] coefficients of a stage written by the
-    // service warp; slot / buffer b = stage mod 2
-    uint64_t *full = reinterpret_cast<uint64_t *>(coef + 64);
-    uint64_t *sums = full + 2, *coefb = full + 4;
-    float4 *tail = reinterpret_cast<float4 *>(full + 6);  // [3][nch - 5 kStepConsumers]
-    const bool has_tail = VM > 5 && p.st_vm3 > 5;   // only with R = 1 and nch > 2400
+    float4 *wsum = reinterpret_cast<float4 *>(ring + p.st_region);    // [kBuf][32]
+    float4 *coef = wsum + 32 * kBuf;                                     // [kBuf][32]
+    // mbarriers: full[NS] ring slot loaded (bulk-copy bytes; slot = stage mod NS), sums[kBuf]
+    // row sums of a stage written by every consumer thread, coefb[kBuf] coefficients of a
+    // stage written by a service warp (buffer b = stage mod kBuf)
+    uint64_t *full = reinterpret_cast<uint64_t *>(coef + 32 * kBuf);
+    uint64_t *sums = full + kStepSlots, *coefb = sums + kBuf;
+    double *svc = reinterpret_cast<double *>(coefb + kBuf);  // [4] second service warp's sums
+    float4 *tail = reinterpret_cast<float4 *>(svc + 4);      // [3][nch - 5 kStepConsumers]
+    const bool has_tail = ONE && VM > 5 && nch > 5 * kStepConsumers;
     const int ntail = has_tail ? nch - 5 * kStepConsumers : 0;
     for (int i = threadIdx.x; i < 3 * ntail; i += blockDim.x) tail[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (threadIdx.x == 0) {
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&full[b], 1);
-            mbar_init(&sums[b], kStepConsumers);
+        for (int b = 0; b < NS; ++b) mbar_init(&full[b], 1);
+        for (int b = 0; b < kBuf; ++b) {
+            mbar_init(&sums[b], nc);
             mbar_init(&coefb[b], 32);
         }
         fence_mbar_init();
@@ -231,21 +248,21 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
 
     bool timed_out = false;
     const uint32_t row_bytes = (uint32_t)ld * sizeof(float);
-    // bulk copy of the rows of stage i into ring slot i mod 2 (one lane of the service warp)
+    // bulk copy of the rows of stage i into ring slot i mod NS (one lane of the service warp)
     auto load_stage = [&](int i) {
         const long long base = r0 + (long long)i * R;
         const uint32_t rows = (uint32_t)min((long long)R, r1 - base);
-        uint64_t *bar = &full[i & 1];
+        const int slot = i % NS;
+        uint64_t *bar = &full[slot];
         mbar_arrive_expect_tx(bar, rows * row_bytes);
-        bulk_g2s(ring + (size_t)(i & 1) * slot_floats, ws.row(s, base), rows * row_bytes, bar);
+        bulk_g2s(ring + slot * slot_floats, ws.row(s, base), rows * row_bytes, bar);
     };
 
-    if (warp == kStepWarps) {
-        // ---------------- the service warp: ring loads and P2 ----------------
-        if (!terminal && lane == 0) {
-            if (nst > 0) load_stage(0);
-            if (nst > 1) load_stage(1);
-        }
+    if (warp >= nc / 32) {
+        // ---------------- a service warp: ring loads and P2 ----------------
+        const int sw = warp - nc / 32;
+        if (!terminal && sw == 0 && lane == 0)
+            for (int i = 0; i < min(NS, nst); ++i) load_stage(i);
         const int PW = T >= 32 ? T >> 5 : 1;          // partial sums per row
         const double t_k = p.level * p.dt;
         const double rho_ref = p.sigma * p.sigma * p.d * t_k;
@@ -254,18 +271,21 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
         const float acs = (float)(2.0 - 0.5 * p.sigma * p.sigma);
         const double lc_d = (2.0 + p.d) / (2.0 * p.d);
         const float lc_f = (float)lc_d;
-        const double yref = terminal ? st.gx0 : st.alpha;
+        const double alpha = terminal ? 0.0 : st.alpha, yref = terminal ? st.gx0 : alpha;
         const double feat_level = terminal ? 0.0 : f_feature(p, t_k, 0.0, st.sumz, st.zz);
         const bool cos_g = p.kind == FBSDE_AC_MANUFACTURED || p.kind == FBSDE_COS_LINEAR_TEST;
         double accW = 0.0, accC = 0.0, accR = 0.0;
         int it_max = 0, failed = 0;
-        for (int i = 0; i < nst; ++i) {
-            const int b = i & 1;
+        for (int i = sw; i < nst; i += kService) {
+            const int b = i & (kBuf - 1);
             const long long base = r0 + (long long)i * R;
             const int nrows = (int)min((long long)R, r1 - base);
-            mbar_wait_or_flag(&sums[b], (uint32_t)((i >> 1) & 1), timed_out);
-            // the consumers are done with slot i mod 2: refill it with stage i + 2
-            if (!terminal && lane == 0 && i + 2 < nst) load_stage(i + 2);
+            mbar_wait_or_flag(&sums[b], (uint32_t)((i / kBuf) & 1), timed_out);
+            // one row per stage: the consumers are done with the slot of stage i (its column
+            // pass reads the row back from L2); several: with that of the last stage whose
+            // column pass came before this stage's sums.  Refill it.
+            const int freed = ONE ? i : i - LAG - 1;
+            if (!terminal && lane == 0 && freed >= 0 && freed + NS < nst) load_stage(freed + NS);
             if (lane < nrows) {
                 const long long j = base + lane;
                 float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
@@ -292,7 +312,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
                         feat_d = (double)feat_f;
                     }
                     int it;
-                    Yj = newton_fp32_fp64(p, st.alpha + (double)a0, feat_f, feat_d, lc_f, lc_d, it);
+                    Yj = newton_fp32_fp64(p, alpha + (double)a0, feat_f, feat_d, lc_f, lc_d, it);
                     if (it < 0) {
                         failed = 1;
                         it = p.newton_max_iter;
@@ -324,16 +344,32 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             it_max = max(it_max, __shfl_xor_sync(0xffffffffu, it_max, o));
         }
         const bool any_failed = __any_sync(0xffffffffu, failed);
-        if (!terminal && lane == 0) {   // every copy issued has landed before the CTA exits
-            for (int i = max(0, nst - 2); i < nst; ++i)
-                mbar_wait_or_flag(&full[i & 1], (uint32_t)((i >> 1) & 1), timed_out);
+        // every copy issued has landed before the CTA exits (with several rows per stage the
+        // consumers have waited for each)
+        if (ONE && !terminal && lane == 0)
+            for (int i = max(0, nst - NS); i < nst; ++i)
+                mbar_wait_or_flag(&full[i % NS], (uint32_t)((i / NS) & 1), timed_out);
+        if (!ONE) {   // the first warp adds the second's sums
+            if (sw == 1 && lane == 0) {
+                svc[0] = accW;
+                svc[1] = accC;
+                svc[2] = accR;
+            }
+            bar_named(kStepBarSum, 64);
+            if (sw == 0) {
+                accW += svc[0];
+                accC += svc[1];
+                accR += svc[2];
+            }
         }
         if (timed_out) atomicCAS(&st.status, 0, (int)FBSDE_ERR_TIMEOUT);
         if (lane == 0) {
-            double *o = ws.spart(s, g);
-            o[0] = accW;
-            o[1] = accC;
-            o[2] = accR;
+            if (sw == 0) {
+                double *o = ws.spart(s, g);
+                o[0] = accW;
+                o[1] = accC;
+                o[2] = accR;
+            }
             if (!terminal) {
                 if (it_max) {
                     atomicMax(&st.newton_max, it_max);
@@ -347,10 +383,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
 
     // ---------------- consumers: P1 and P3 ----------------
     const int ct = threadIdx.x;                 // 0 .. kStepConsumers - 1
-    const int team = ONE ? 0 : ct / T, tl0 = ONE ? ct : ct - team * T;
-    const int tpr = ONE ? kStepConsumers : p.st_tpr, RG = ONE ? 1 : p.st_RG;
-    const int vm3 = ONE ? VM : p.st_vm3;
-    const int rg = ONE ? 0 : ct / tpr, tc = ONE ? ct : ct - rg * tpr;
+    const int team = ONE ? 0 : ct / T, tl = ONE ? ct : ct - team * T;
     const float wa = (float)p.wa, wb = (float)p.wb;
     const uint32_t kk = (uint32_t)p.level;
     // chunk v = tl + T v of a row exists (ONE: every v < VM - 1 does)
@@ -359,11 +392,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
 #pragma unroll
     for (int v = 0; v < VMR; ++v)
         acc[0][v] = acc[1][v] = acc[2][v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    // HELD: the chunks this thread stepped in the stage before and in this one; chunks past
-    // the row stay 0, rows past the stage are masked by their coefficients
-    float4 prev[HELD ? VM : 1], cur[HELD ? VM : 1];
-#pragma unroll
-    for (int v = 0; v < (HELD ? VM : 1); ++v) prev[v] = cur[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     // fma of one chunk of a row into the three accumulators of chunk v
     auto acc3 = [&](float4 (&a)[3], const float4 cf, const float4 x) {
         const float2 xl = lo2(x), xh = hi2(x);
@@ -379,7 +407,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
         a[2] = make_float4(l.x, l.y, h.x, h.y);
     };
     auto p3 = [&](int i) {
-        const int b = i & 1;
+        const int b = i & (kBuf - 1);
         const long long base = r0 + (long long)i * R;
         const int nrows = ONE ? 1 : (int)min((long long)R, r1 - base);
         if (ONE) {
@@ -391,21 +419,21 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             float4 x[VM];
 #pragma unroll
             for (int v = 0; v < VM; ++v) {
-                const int c = tc + tpr * v;
+                const int c = tl + T * v;
                 if (in_row(v, c)) x[v] = __ldcg(row + c);
             }
-            mbar_wait_or_flag(&coefb[b], (uint32_t)((i >> 1) & 1), timed_out);
+            mbar_wait_or_flag(&coefb[b], (uint32_t)((i / kBuf) & 1), timed_out);
             const float4 cf = coef[b * 32];
 #pragma unroll
             for (int v = 0; v < VMR; ++v) {
                 float4 a[3] = {acc[0][v], acc[1][v], acc[2][v]};
-                if (in_row(v, tc + tpr * v)) acc3(a, cf, x[v]);
+                if (in_row(v, tl + T * v)) acc3(a, cf, x[v]);
                 acc[0][v] = a[0];
                 acc[1][v] = a[1];
                 acc[2][v] = a[2];
             }
             if (VM > 5 && has_tail) {
-                const int c = tc + tpr * 5;
+                const int c = tl + T * 5;
                 if (c < nch) {
                     float4 *t0 = tail + (c - 5 * kStepConsumers);
                     float4 a[3] = {t0[0], t0[ntail], t0[2 * ntail]};
@@ -417,51 +445,35 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             }
             return;
         }
-        mbar_wait_or_flag(&coefb[b], (uint32_t)((i >> 1) & 1), timed_out);
-        if constexpr (HELD) {   // the team's own row, from registers
-            if (team < nrows) {
-                const float4 cf = coef[b * 32 + team];
+        mbar_wait_or_flag(&coefb[b], (uint32_t)((i / kBuf) & 1), timed_out);
+        if (team < nrows) {   // this thread's own chunks, left in the ring by P1
+            const float4 cf = coef[b * 32 + team];
+            const float4 *sl = reinterpret_cast<const float4 *>(ring + (i % NS) * slot_floats +
+                                                                (size_t)team * ld);
 #pragma unroll
-                for (int v = 0; v < VMR; ++v) {
+            for (int v = 0; v < VMR; ++v) {
+                const int c = tl + T * v;
+                if (c < nch) {
                     float4 a[3] = {acc[0][v], acc[1][v], acc[2][v]};
-                    acc3(a, cf, prev[v]);
+                    acc3(a, cf, sl[c]);
                     acc[0][v] = a[0];
                     acc[1][v] = a[1];
                     acc[2][v] = a[2];
-                }
-            }
-            return;
-        }
-        if (rg < RG) {
-            for (int r = rg; r < nrows; r += RG) {
-                const float4 cf = coef[b * 32 + r];
-                // the row stepped in P1 of stage i, read back through L2
-                const float4 *row = reinterpret_cast<const float4 *>(ws.row(s, base + r));
-#pragma unroll
-                for (int v = 0; v < VMR; ++v) {
-                    const int c = tc + tpr * v;
-                    if (v < vm3 && c < nch) {
-                        float4 a[3] = {acc[0][v], acc[1][v], acc[2][v]};
-                        acc3(a, cf, __ldcg(row + c));
-                        acc[0][v] = a[0];
-                        acc[1][v] = a[1];
-                        acc[2][v] = a[2];
-                    }
                 }
             }
         }
     };
 
     for (int i = 0; i < nst; ++i) {
-        const int b = i & 1;
+        const int b = i & (kBuf - 1), slot = i % NS;
         const long long base = r0 + (long long)i * R;
         const int nrows = ONE ? 1 : (int)min((long long)R, r1 - base);
         const bool active = ONE || team < nrows;
-        const int tl = tl0;
         const long long j = base + team;
         float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
         float2 q0 = make_float2(0.f, 0.f), q1 = q0, q3 = q0;   // pair sums of the level step
         float4 *dst = reinterpret_cast<float4 *>(ws.row(s, active ? j : base));
+        float4 *sl = reinterpret_cast<float4 *>(ring + slot * slot_floats + (size_t)team * ld);
         if (terminal) {
             if (active) {
                 const int kind = p.kind;
@@ -495,14 +507,12 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
                                                            : s1 + ((tx.x + tx.y) + (tx.z + tx.w));
                         }
                         dst[c] = z;
-                        if (HELD) cur[HELD ? v : 0] = z;
+                        if (!ONE) sl[c] = z;
                     }
                 }
             }
         } else {
-            mbar_wait_or_flag(&full[b], (uint32_t)((i >> 1) & 1), timed_out);
-            const float4 *sl = reinterpret_cast<const float4 *>(ring + (size_t)b * slot_floats +
-                                                                (size_t)team * ld);
+            mbar_wait_or_flag(&full[slot], (uint32_t)((i / NS) & 1), timed_out);
             if (active) {
 #pragma unroll
                 for (int v = 0; v < VM; ++v) {
@@ -531,7 +541,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
                             s2 += (cos_ftz(xa.x) + cos_ftz(xa.y)) + (cos_ftz(xb.x) + cos_ftz(xb.y));
                         }
                         dst[c] = dn;
-                        if (HELD) cur[HELD ? v : 0] = dn;
+                        if (!ONE) sl[c] = dn;
                     }
                 }
             }
@@ -552,28 +562,39 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             }
             if ((lane & 15) == 0) wsum[b * 32 + (ct >> 4)] = make_float4(s0, s1, s2, s3);
         }
+        if (!ONE && !terminal) fence_async_smem();   // before the slot's next copy
         mbar_arrive(&sums[b]);
-        if (i >= 1) p3(i - 1);
-        if (HELD) {
-#pragma unroll
-            for (int v = 0; v < (HELD ? VM : 1); ++v) prev[v] = cur[v];
-        }
+        if (i >= LAG) p3(i - LAG);
     }
-    if (nst >= 1) p3(nst - 1);
+    for (int i = max(0, nst - LAG); i < nst; ++i) p3(i);
     if (timed_out) atomicCAS(&st.status, 0, (int)FBSDE_ERR_TIMEOUT);
 
-    if constexpr (HELD) {   // the teams' sums, added in team order
-        bar_named(kStepBarEnd, kStepConsumers);   // every consumer is past its last ring read
+    if constexpr (ONE) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            float4 *dst = reinterpret_cast<float4 *>(ws.part(s, g, a));
+#pragma unroll
+            for (int v = 0; v < VMR; ++v) {
+                const int c = tl + T * v;
+                if (in_row(v, c)) dst[c] = acc[a][v];
+            }
+            if (VM > 5 && has_tail) {
+                const int c = tl + T * 5;
+                if (c < nch) dst[c] = tail[a * ntail + (c - 5 * kStepConsumers)];
+            }
+        }
+    } else {   // the teams' sums, added in team order
+        bar_named(kStepBarEnd, nc);   // every consumer is past its last ring read
         float4 *red = reinterpret_cast<float4 *>(ring);   // [R][3][nch]
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int v = 0; v < VMR; ++v) {
-                const int c = tl0 + T * v;
+                const int c = tl + T * v;
                 if (c < nch) red[((size_t)team * 3 + a) * nch + c] = acc[a][v];
             }
-        bar_named(kStepBarEnd, kStepConsumers);
-        for (int idx = ct; idx < 3 * nch; idx += kStepConsumers) {
+        bar_named(kStepBarEnd, nc);
+        for (int idx = ct; idx < 3 * nch; idx += nc) {
             const int a = idx / nch, c = idx - a * nch;
             float4 sum = red[(size_t)a * nch + c];
             for (int r = 1; r < R; ++r) {
@@ -585,46 +606,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(Params p)
             }
             reinterpret_cast<float4 *>(ws.part(s, g, a))[c] = sum;
         }
-        return;
-    }
-    // per-CTA partial d-vectors: row groups summed in group order (threads past the RG
-    // row groups of tpr threads own no chunk)
-    if (RG == 1) {
-        if (rg >= RG) return;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            float4 *dst = reinterpret_cast<float4 *>(ws.part(s, g, a));
-#pragma unroll
-            for (int v = 0; v < VMR; ++v) {
-                const int c = tc + tpr * v;
-                if (v < vm3 && in_row(v, c)) dst[c] = acc[a][v];
-            }
-            if (VM > 5 && has_tail) {
-                const int c = tc + tpr * 5;
-                if (c < nch) dst[c] = tail[a * ntail + (c - 5 * kStepConsumers)];
-            }
-        }
-        return;
-    }
-    bar_named(kStepBarEnd, kStepConsumers);   // every consumer is past its last ring read
-    float4 *red = reinterpret_cast<float4 *>(ring);   // [RG][3][nch]
-    if (rg < RG) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (tc < nch) red[((size_t)rg * 3 + a) * nch + tc] = acc[a][0];
-    }
-    bar_named(kStepBarEnd, kStepConsumers);
-    for (int idx = ct; idx < 3 * nch; idx += kStepConsumers) {
-        const int a = idx / nch, c = idx - a * nch;
-        float4 sum = red[(size_t)a * nch + c];
-        for (int r = 1; r < RG; ++r) {
-            const float4 o = red[((size_t)r * 3 + a) * nch + c];
-            sum.x += o.x;
-            sum.y += o.y;
-            sum.z += o.z;
-            sum.w += o.w;
-        }
-        reinterpret_cast<float4 *>(ws.part(s, g, a))[c] = sum;
     }
 }
 

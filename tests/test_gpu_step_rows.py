@@ -1,5 +1,5 @@
-"""The fused level step at the edges of the form whose column pass takes the stepped chunks from
-the row pass's registers: four and five chunks per thread at 30, 15, 5 and 3 rows per stage, and
+"""The fused level step where its geometry changes: rows per stage from 32 down to one, one to
+five chunks per thread, rings of three to eight stages with either lag of the column pass, and
 small clouds spread over one wave of CTAs, against the FP64 oracle (FP32 bar 1e-4)."""
 import pytest
 
@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
                                         ("ac_manufactured", 1536, 2141, 1),
                                         ("logistic_grad", 1537, 2003, 1),
                                         ("ac_manufactured", 2560, 3201, 1),
+                                        ("logistic_grad", 3412, 3607, 1),
+                                        ("ac_manufactured", 3416, 3601, 1),
                                         ("ac_manufactured", 50, 3001, 1),
                                         ("logistic_grad", 340, 457, 3)])
 def test_step_rows_match_oracle(kind, d, M, Q):
