@@ -252,8 +252,9 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     // holds five (it frees a slot lag + 1 stages after its row pass, and a slot is requested
     // at least one stage ahead), else one.
     L.sde = is_sde(P) ? 1 : 0;
-    L.fused = !L.sde && P->precision == FBSDE_FP32 && L.ld <= kStepMaxLd;
-    if (L.fused) {
+    const bool step = P->precision == FBSDE_FP32 && L.ld <= kStepMaxLd;
+    L.fused = !L.sde && step;
+    if (step) {
         L.st_R = 1;
         L.st_T = 480;
         double best_rate = 0.0;
@@ -284,9 +285,10 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
             return FBSDE_ERR_ARG;
     }
     // CTAs per query of the fused step (one CTA per SM): whole waves of 152 CTAs where
-    // possible, at least four stages per CTA; 4..1 waves first, then 5..8
+    // possible, at least four stages per CTA; 4..1 waves first, then 5..8.  (Also for a
+    // forward SDE, which has no such step: its partial vectors' buffer is the same.)
     L.Gs = L.G;
-    if (L.fused) {
+    if (step) {
         const long long gmax_s = std::max<long long>(1, P->M / (4LL * L.st_R));
         // a cloud too small for that on every SM takes one wave of CTAs with fewer stages
         // (d = 64, M = 512: 17 CTAs of one stage in place of 4 of four,
