@@ -118,8 +118,9 @@ typedef struct {
     double newton_tol;       /* Newton stops when |dY| <= newton_tol max(1,|Y|); 0 selects 1e-13 */
     int32_t ctas;            /* CTAs of one streaming pass over all Q queries (tiling of the
                                 particle clouds; results depend on it through the order of
-                                the partial sums); 0 selects 608; at most M / 32 CTAs
-                                per query are used                                       */
+                                the partial sums); 0 selects 608, and for the CG's
+                                products as many whole waves of one per SM as divide
+                                the rows best; else at most M / 32 CTAs per query        */
     int32_t reserved;        /* must be 0                                               */
     /* Forward SDE dX = mu(t,X) dt + sigma(t,X) dW of Sec. 2.1 with the componentwise affine
        coefficients mu_i(x) = mu0 + mu1 x_i and sigma(x) = diag(sigma + sig1 x_i).  With
@@ -343,9 +344,10 @@ FBSDE_API int fbsde_normals(uint64_t seed, uint32_t s, uint32_t k, uint32_t j0, 
 /*
  * Plans: a solve, or a batch of heterogeneous solves (each Algorithm 1 on its own problem,
  * query points and cloud; the batching itself has no counterpart in the paper), captured
- * once into a CUDA graph and replayed with one launch.  Each CG loop is a conditional while node whose body
- * (product, reduction, CG step, convergence check) repeats on the device until every
- * query of that instance has converged, so no empty iterations are launched.  Instances
+ * once into a CUDA graph and replayed with one launch.  Each CG loop stops on the device when
+ * every query of that instance has converged, so no empty iterations are launched: one
+ * cooperative launch per loop in a plan of one branch, else a conditional while node whose
+ * body (product, vector updates, convergence check) repeats.  Instances
  * are spread over parallel graph branches and run concurrently on the GPU.  The
  * pointers of every instance are bound at creation: refill x0 in place and launch again.
  */
@@ -421,8 +423,9 @@ typedef struct {
    family, the first FBSDE_PROFILED_EAGER_PASSES passes of every loop are launched one by
    one (each product launch bracketed by events; kernels of converged queries exit at
    once) and any further passes run in a cached CUDA graph whose conditional while loop
-   stops when every query has converged.  Otherwise every pass runs in that graph.  On a
-   stream that is being captured every pass is launched one by one, up to cg_max_iter.
+   stops when every query has converged.  Otherwise every pass of a loop runs in one
+   cooperative launch, or, for the shapes that it does not serve, in that graph.  On a
+   stream that is being captured these are launched one by one, up to cg_max_iter passes.
    The results are the same bit for bit in every case. */
 #define FBSDE_PROFILED_EAGER_PASSES 48
 FBSDE_API int fbsde_profile_start(int32_t max_timed_launches);

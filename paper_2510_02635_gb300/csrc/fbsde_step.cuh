@@ -35,8 +35,8 @@
 // after stage bounded the kernel for narrow rows: d = 1000, 64 queries of 4096 particles,
 // five rows a stage, 823 us a level with one service warp (596 us with its Newton iterations
 // left out), 699 us with two of them and a lag of two stages, 620 us with nine rows and 18
-// consumer warps (663 us with 15).  Against 4.2 GB read and written that is 3.4 TB/s; the
-// issue of the normals' arithmetic (43 instructions per particle-dim) bounds it now.
+// consumer warps (663 us with seven and 14).  That is 3.4 TB/s read and written; it is bound by issue
+// now (65% of the issue slots at 20 warps an SM, the normals' arithmetic first).
 // Hand-offs by mbarriers: sums[b] "stage i stepped: row sums written" (every consumer arrives,
 // the service warp waits), coefb[b] "coefficients of stage i ready" (the service warp arrives,
 // each consumer waits on its own), so the consumer warps never wait for one another and a fast
