@@ -291,8 +291,8 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     if (step) {
         const long long gmax_s = std::max<long long>(1, P->M / (4LL * L.st_R));
         // a cloud too small for that on every SM takes one wave of CTAs with fewer stages
-        // (d = 64, M = 512: 17 CTAs of one stage in place of 4 of four,
-        // 16.6 -> 7.7 us a level)
+        // (d = 64, M = 512: 18 CTAs of one stage in place of 4 of four,
+        // 16.6 -> 7.9 us a level)
         const long long gone = std::max<long long>(gmax_s, (P->M + L.st_R - 1) / L.st_R);
         double best = -1.0;
         for (int W : {4, 3, 2, 1, 5, 6, 7, 8}) {

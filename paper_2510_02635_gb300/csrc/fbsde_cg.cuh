@@ -509,7 +509,7 @@ struct CgProducer {
 // the reads of r, of the partials and of the shares (0.5 to 1 us each through L2), and two
 // chains of dependent FP64 operations (64 cycles each).  Measured with one query: d = 1000,
 // M = 4096, 8.6 us a pass in place of 20.5 us in three launches; d = 2503, M = 8192, 21 us
-// (82 MB of rows, phase A 12 us) in place of 43 us; FP64, d = 1203, M = 2048, 26 us in place
+// (82 MB of rows, phase A 12 us) in place of 43 us; FP64, d = 1203, M = 2048, 23 us in place
 // of 63 us (the product had 64 CTAs).  Warp 0 polls the barrier; the first loads a warp makes
 // after its polls take 4 us longer (measured on 80 of the 152 SMs), so it takes no part in
 // phase B and the scalars fall to the last warp.
