@@ -288,30 +288,30 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     // possible, at least four stages per CTA; 4..1 waves first, then 5..8.  (Also for a
     // forward SDE, which has no such step: its partial vectors' buffer is the same.)
     L.Gs = L.G;
-    if (step) {
+    auto step_ctas = [&](long long most) {
+        int Gs = L.G;
         const long long gmax_s = std::max<long long>(1, P->M / (4LL * L.st_R));
         // a cloud too small for that on every SM takes one wave of CTAs with fewer stages
         // (d = 64, M = 512: 18 CTAs of one stage in place of 4 of four,
-        // 16.6 -> 7.9 us a level)
-        const long long gone = std::max<long long>(gmax_s, (P->M + L.st_R - 1) / L.st_R);
+        // 16.6 -> 7.9 us a level), three rows at least: its partial vectors (three a CTA)
+        // take no more room than the rows
+        const long long gone =
+            std::max<long long>(gmax_s, std::min((P->M + L.st_R - 1) / L.st_R, P->M / 3));
         double best = -1.0;
         for (int W : {4, 3, 2, 1, 5, 6, 7, 8}) {
-            const long long g = std::min<long long>(W == 1 && gmax_s * Q < 152 ? gone : gmax_s,
-                                                    (152LL * W + Q - 1) / Q);
+            const long long g = std::min<long long>({W == 1 && gmax_s * Q < 152 ? gone : gmax_s,
+                                                     (152LL * W + Q - 1) / Q, most});
             const double waves = (double)(g * Q) / 152.0;
             const double eff = waves / std::ceil(waves);
             if (eff > best + 1e-9) {
                 best = eff;
-                L.Gs = (int)g;
+                Gs = (int)g;
             }
             if (eff >= 0.99) break;
         }
-    }
-    if (!cg_geometry(P, Q, L)) return FBSDE_ERR_ARG;
-    product_ring(P, (size_t)L.ld * L.real_sz, L.Gc, L.teams, L.real_sz, L.mv_rows, L.mv_stages,
-                 L.mv_smem);
-    if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
-    L.GS = std::max(L.GP, L.fused ? L.Gs : 0);
+        return Gs;
+    };
+    if (step) L.Gs = step_ctas(P->M);
     // partial reduction: tiles of kRedTile elements, red_groups warps per tile, each adding
     // about four of the G partials
     L.nblk = (L.ld + kRedTile - 1) / kRedTile;
@@ -319,37 +319,60 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     // moments: column tiles of 256 * mom_vm chunks
     L.mom_vm = nch > 256 ? 2 : 1;
     L.mom_tiles = (nch + 256 * L.mom_vm - 1) / (256 * L.mom_vm);
+    const size_t Qs = (size_t)Q, Ms = (size_t)P->M, lds = (size_t)L.ld;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off = align_up(off + bytes, kAlign);
         return o;
     };
-    const size_t Qs = (size_t)Q, Ms = (size_t)P->M, lds = (size_t)L.ld;
-    L.off_delta = take(Qs * Ms * lds * L.real_sz);
-    L.off_Y = take(Qs * Ms * sizeof(double));
-    L.off_w = take(Qs * Ms * L.real_sz);
-    L.off_coef = take(Qs * Ms * 3 * L.real_sz);
-    L.off_segp = take(Qs * Ms * (size_t)L.nseg * kSegSums * L.real_sz);
-    L.off_part = take(Qs * std::max(L.G, L.Gs) * kPartVecs * lds * L.real_sz);
-    L.off_spart = take(Qs * L.GS * kPartScal * sizeof(double));
-    L.off_vec64 = take(Qs * kVec64 * lds * sizeof(double));
-    L.off_vecR = take((Qs * kVecR + 1) * lds * L.real_sz);
-    L.off_state = take(Qs * sizeof(SolveState));
-    L.off_bpart = take(Qs * (size_t)L.nblk * kBpart * sizeof(double));
-    if (L.sde) {
-        // Euler-Maruyama rows: checkpoints at the levels s, 2s, .. below N and one segment of
-        // s - 1 levels, s = ceil(sqrt N): about 2 sqrt(N) slabs of Q M ld instead of N - 1,
-        // for one more forward step per level on the way back
-        int sq = 1;
-        while (sq * sq < P->N) ++sq;
-        L.sde_s = sq;
-        L.sde_ncp = (P->N - 1) / sq;
-        L.sde_slots = L.sde_ncp + sq - 1;
-        L.off_store = take((size_t)L.sde_slots * Qs * Ms * lds * L.real_sz);
-        L.off_anchor = take(Qs * (size_t)(P->N + 1) * lds * L.real_sz);
+    auto place = [&] {
+        off = 0;
+        L.GS = std::max(L.GP, L.fused ? L.Gs : 0);
+        L.off_delta = take(Qs * Ms * lds * L.real_sz);
+        L.off_Y = take(Qs * Ms * sizeof(double));
+        L.off_w = take(Qs * Ms * L.real_sz);
+        L.off_coef = take(Qs * Ms * 3 * L.real_sz);
+        L.off_segp = take(Qs * Ms * (size_t)L.nseg * kSegSums * L.real_sz);
+        L.off_part = take(Qs * std::max(L.G, L.Gs) * kPartVecs * lds * L.real_sz);
+        L.off_spart = take(Qs * L.GS * kPartScal * sizeof(double));
+        L.off_vec64 = take(Qs * kVec64 * lds * sizeof(double));
+        L.off_vecR = take((Qs * kVecR + 1) * lds * L.real_sz);
+        L.off_state = take(Qs * sizeof(SolveState));
+        L.off_bpart = take(Qs * (size_t)L.nblk * kBpart * sizeof(double));
+        if (L.sde) {
+            // Euler-Maruyama rows: checkpoints at the levels s, 2s, .. below N and one segment
+            // of s - 1 levels, s = ceil(sqrt N): about 2 sqrt(N) slabs of Q M ld instead of
+            // N - 1, for one more forward step per level on the way back
+            int sq = 1;
+            while (sq * sq < P->N) ++sq;
+            L.sde_s = sq;
+            L.sde_ncp = (P->N - 1) / sq;
+            L.sde_slots = L.sde_ncp + sq - 1;
+            L.off_store = take((size_t)L.sde_slots * Qs * Ms * lds * L.real_sz);
+            L.off_anchor = take(Qs * (size_t)(P->N + 1) * lds * L.real_sz);
+        }
+        L.total = off;
+    };
+    place();
+    // The step's partial vectors alone never put a problem beyond the fixed scratch of
+    // fbsde_solve_noalloc: where those of the other passes' L.G CTAs would fit, the step takes
+    // no more CTAs than do (every entry point has the same tiling).
+    if (L.Gs > L.G && L.total > (size_t)FBSDE_NOALLOC_MAX_BYTES) {
+        const int most = L.Gs;
+        L.Gs = L.G;
+        place();
+        if (L.total + 2 * kAlign <= (size_t)FBSDE_NOALLOC_MAX_BYTES)
+            L.Gs = step_ctas(L.G + (FBSDE_NOALLOC_MAX_BYTES - 2 * kAlign - L.total) /
+                                       (Qs * kPartVecs * lds * L.real_sz + Qs * kPartScal * 8));
+        else if (L.total > (size_t)FBSDE_NOALLOC_MAX_BYTES)
+            L.Gs = most;
+        place();
     }
-    L.total = off;
+    if (!cg_geometry(P, Q, L)) return FBSDE_ERR_ARG;
+    product_ring(P, (size_t)L.ld * L.real_sz, L.Gc, L.teams, L.real_sz, L.mv_rows, L.mv_stages,
+                 L.mv_smem);
+    if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
     // reverse sweep: tape of the primal plus three adjoint vectors per query
     L.off_tape_w = take((size_t)P->N * Qs * Ms * L.real_sz);
     L.off_tape_Y = take((size_t)(P->N + 1) * Qs * Ms * sizeof(double));
