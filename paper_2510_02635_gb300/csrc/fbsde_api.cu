@@ -8,6 +8,8 @@
 #include <numeric>
 #include <vector>
 
+#include <cuda.h>
+
 #include "fbsde_kernels.cuh"
 #include "fbsde_cg.cuh"
 #include "fbsde_matvec.cuh"
@@ -530,6 +532,48 @@ struct Rec {
     int branches = 1;
 };
 
+}  // namespace
+
+// The SMs of the device, or fewer where the stream (or the calling thread's context) belongs to
+// a green context, whose kernels run on its own SMs only.  The driver's functions are looked up
+// by name, so that the library needs no link against it; the stream's part is read on each call.
+int coop_sms(cudaStream_t s)
+{
+    int dev = 0, n = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    struct Driver {
+        decltype(&cuStreamGetGreenCtx) green = nullptr;
+        decltype(&cuGreenCtxGetDevResource) resource = nullptr;
+        Driver()
+        {
+            auto find = [](const char *name) -> void * {
+                void *f = nullptr;
+                cudaDriverEntryPointQueryResult q;
+                if (cudaGetDriverEntryPointByVersion(name, &f, 12050, cudaEnableDefault, &q) !=
+                        cudaSuccess || q != cudaDriverEntryPointSuccess) {
+                    (void)cudaGetLastError();
+                    return nullptr;
+                }
+                return f;
+            };
+            green = reinterpret_cast<decltype(green)>(find("cuStreamGetGreenCtx"));
+            resource = reinterpret_cast<decltype(resource)>(find("cuGreenCtxGetDevResource"));
+        }
+    };
+    static const Driver drv;
+    CUgreenCtx g = nullptr;
+    CUdevResource res{};
+    if (drv.green && drv.resource && drv.green(s, &g) == CUDA_SUCCESS && g &&
+        drv.resource(g, &res, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+        n = std::min(n, (int)res.sm.smCount);
+    return n;
+}
+
+namespace {
+
 // The parameters as the CG's kernels see them: the product's chunks, one vector per partial.
 Params product_params(const Params &p, const Layout &L)
 {
@@ -684,43 +728,51 @@ template <typename Real> cudaError_t cg_graph_launch(const Params &p, const Layo
 }
 
 // The CG iterations of one regression (all queries of the launch together): one cooperative
-// launch of the whole loop wherever the shape has one and the work does not share the GPU
-// with other branches of a plan.  Otherwise a conditional while loop of the two phases:
-// captured into the plan's graph, or (graph_tail) a cached CUDA graph, or, on a stream that
-// is itself being captured and without graph_tail, every pass launched one by one (kernels
-// of queries that have converged exit at once).  While the launch profiler times the product
-// kernel, the first kEagerPasses passes are launched one by one so that their products can
-// be bracketed by events.  Every form gives the same bits.
+// launch of the whole loop wherever the shape has one, the stream's SMs take it and the work
+// does not share the GPU with other branches of a plan.  Otherwise (also where the driver finds
+// the cooperative launch too large) a conditional while loop of the two phases: captured into
+// the plan's graph, or (graph_tail) a cached CUDA graph, or, on a stream that is itself being
+// captured and without graph_tail, every pass launched one by one (kernels of queries that have
+// converged exit at once).  While the launch profiler times the product kernel, the first
+// kEagerPasses passes are launched one by one so that their products can be bracketed by
+// events.  Every form gives the same bits.
 template <typename Real> cudaError_t cg_loop(const Params &p0, const Layout &L, const Rec &r)
 {
     using LR = Launch<Real>;
     cudaError_t e;
     const cudaStream_t s = r.s;
     const Params p = product_params(p0, L);
-    const bool one = r.branches == 1 && !L.cg3 && LR::cg_loop_fits(L);
-    if (r.capture) return one ? LR::cg_loop(p, L, s) : cg_capture<Real>(p, L, s, r.body);
-    bool tail = r.graph_tail || one;
-    if (tail && !one) {
+    const bool one = r.branches == 1 && !L.cg3 && LR::cg_loop_fits(L, s);
+    int pass = 0;
+    auto passes = [&](int upto) -> cudaError_t {
+        for (; pass < upto; ++pass) {
+            if (L.cg3) {
+                FBSDE_TRY(FBSDE_K_MATVEC, LR::cg3(p, L, 0, 0, 0, s));
+                FBSDE_TRY(FBSDE_K_REDUCE, LR::cg3(p, L, 1, 0, 0, s));
+                FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg3(p, L, 2, 0, 0, s));
+                continue;
+            }
+            FBSDE_TRY(FBSDE_K_MATVEC, LR::matvec(p, L, s));
+            FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_tile(p, L, 0, 0, s));
+        }
+        return cudaSuccess;
+    };
+    const int first = !r.capture && profiling_products() ? std::min(p.cg_max_iter, kEagerPasses) : 0;
+    if (one) {
+        if ((e = passes(first)) != cudaSuccess || pass >= p.cg_max_iter) return e;
+        ProfScope ps(r.capture ? -1 : FBSDE_K_CG_STEP, s);
+        if ((e = LR::cg_loop(p, L, s)) != cudaErrorCooperativeLaunchTooLarge) return e;
+        (void)cudaGetLastError();
+    }
+    if (r.capture) return cg_capture<Real>(p, L, s, r.body);
+    bool tail = r.graph_tail;
+    if (tail) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if ((e = cudaStreamIsCapturing(s, &cs)) != cudaSuccess) return e;
         tail = cs == cudaStreamCaptureStatusNone;
     }
-    const int eager = !tail ? p.cg_max_iter
-                            : (profiling_products() ? std::min(p.cg_max_iter, kEagerPasses) : 0);
-    for (int it = 0; it < eager; ++it) {
-        if (L.cg3) {
-            FBSDE_TRY(FBSDE_K_MATVEC, LR::cg3(p, L, 0, 0, 0, s));
-            FBSDE_TRY(FBSDE_K_REDUCE, LR::cg3(p, L, 1, 0, 0, s));
-            FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg3(p, L, 2, 0, 0, s));
-            continue;
-        }
-        FBSDE_TRY(FBSDE_K_MATVEC, LR::matvec(p, L, s));
-        FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_tile(p, L, 0, 0, s));
-    }
-    if (eager >= p.cg_max_iter) return cudaSuccess;
-    if (!one) return cg_graph_launch<Real>(p, L, s);
-    FBSDE_TRY(FBSDE_K_CG_STEP, LR::cg_loop(p, L, s));
-    return cudaSuccess;
+    if ((e = passes(tail ? first : p.cg_max_iter)) != cudaSuccess || pass >= p.cg_max_iter) return e;
+    return cg_graph_launch<Real>(p, L, s);
 }
 
 template <typename Real>

@@ -36,6 +36,10 @@ int solve_launches_only(const fbsde_problem *P, int32_t Q, const double *x0, uin
                         uint32_t solve_index0, double *u0, double *grad_u0, void *workspace,
                         size_t workspace_bytes, cudaStream_t stream);
 
+// SMs that a cooperative launch on stream s can take, 0 without cooperative launches
+// (fbsde_api.cu).
+int coop_sms(cudaStream_t s);
+
 constexpr int kPartVecs = 3;
 constexpr int kPartScal = 4;
 constexpr int kVec64 = 9;
@@ -165,7 +169,7 @@ template <typename Real> struct Launch {
     // the pass in three launches (0: product, 1: reduction, 2: updates), FP32 only
     static cudaError_t cg3(const Params &p, const Layout &L, int kernel, cudaGraphConditionalHandle h,
                            int use_h, cudaStream_t s);
-    static bool cg_loop_fits(const Layout &L);   // on the current device
+    static bool cg_loop_fits(const Layout &L, cudaStream_t s);
     static cudaError_t cg_loop(const Params &p, const Layout &L, cudaStream_t s);
     static cudaError_t cg_post(const Params &p, const Layout &L, cudaStream_t s);
     // the same per level over tiles (fbsde_level.cuh)

@@ -301,17 +301,6 @@ cudaError_t Launch<Real>::cg3(const Params &p0, const Layout &L, int kernel,
     }
 }
 
-// SMs of the current device, 0 without cooperative launches.
-static int coop_sms()
-{
-    int dev = 0, n = 0, coop = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 0;
-    return n;
-}
-
 template <typename Real>
 static void *cg_loop_kernel(const Layout &L)
 {
@@ -328,10 +317,10 @@ static void *cg_loop_kernel(const Layout &L)
 }
 
 // A layout that keeps one chunk per CTA in shared memory needs that many CTAs at once.
-template <typename Real> bool Launch<Real>::cg_loop_fits(const Layout &L)
+template <typename Real> bool Launch<Real>::cg_loop_fits(const Layout &L, cudaStream_t s)
 {
     if (!L.cg_ok || !cg_loop_kernel<Real>(L)) return false;
-    const int sms = coop_sms();
+    const int sms = coop_sms(s);
     return sms > 0 && (!L.cg_res || (long long)L.Q * L.Gc <= sms);
 }
 
@@ -339,7 +328,7 @@ template <typename Real>
 cudaError_t Launch<Real>::cg_loop(const Params &p, const Layout &L, cudaStream_t s)
 {
     void *k = cg_loop_kernel<Real>(L);
-    const int sms = coop_sms();
+    const int sms = coop_sms(s);
     if (!k || sms < 1) return cudaErrorNotSupported;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)L.cg_smem);
