@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(kTileThreads) k_adj_setup(Params p, int warm)
     const double *sc = tp.scal(s, k);
     const double lam = sc[0], invW = sc[1];
     const int width = 4 * p.cg_lpr, i = tile * width + t;
+    if (s == 0 && tile == 0 && t == 0) *p.bar = 0u;   // the CG loop's grid barrier
     double a[3] = {0.0, 0.0, 0.0};
     if (t < width && i < p.ld) {
         const double S = tp.S(s, k)[i], x = warm ? ws.v64(s, 0)[i] : 0.0;

@@ -460,8 +460,10 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_tile(Params p, cudaGraphCondi
 // Barrier of all CTAs of a cooperative launch.  The word's low 31 bits count the arrivals
 // and return to 0 with the last one, which flips the top bit (the first CTA adds
 // 2^31 - (n - 1), the others 1).  Bounded wait: false if the other CTAs did not arrive
-// within kWaitNs.
-__device__ __forceinline__ bool grid_barrier(unsigned int *word, int *flag)
+// within limit_ns; the word may then keep a partial count, so the kernel before every loop
+// sets it to 0 (k_level_rhs, k_adj_setup, k_moments_finalize).
+__device__ __forceinline__ bool grid_barrier(unsigned int *word, int *flag,
+                                             unsigned long long limit_ns = kWaitNs)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -477,7 +479,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int *word, int *flag)
             if ((n & 255u) == 0) {
                 const unsigned long long now = globaltimer_ns();
                 if (!t0) t0 = now;
-                else if (now - t0 > kWaitNs) {
+                else if (now - t0 > limit_ns) {
                     ok = 0;
                     break;
                 }
@@ -514,7 +516,8 @@ struct CgProducer {
 // after its polls take 4 us longer (measured on 80 of the 152 SMs), so it takes no part in
 // phase B and the scalars fall to the last warp.
 // Every CTA keeps the scalars of all queries (the shares are added in the same order
-// everywhere), and the step of those whose tiles it owns.
+// everywhere), and the step of those whose tiles it owns.  After a wait that gave up in an
+// earlier launch of the solve the loop ends at once.
 template <typename Real, int VPT, int NT, bool HOLD>
 __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
 {
@@ -523,6 +526,7 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
     __shared__ double dsl[16];
     __shared__ int flag;
     __shared__ CgProducer pr;
+    if (__ldcg(&p.st[0].status) == FBSDE_ERR_TIMEOUT) return;
     const WS<Real> ws(p);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = p.ld / E, S = p.cg_stages, R = p.cg_rows;

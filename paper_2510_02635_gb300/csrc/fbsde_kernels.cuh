@@ -1213,7 +1213,6 @@ __global__ void __launch_bounds__(kFinThreads) k_setup(Params p, const double *x
         st.gx0 = g_value(p, phi);
         st.yref = st.gx0;
         p.st[s] = st;
-        if (s == 0) *p.bar = 0u;   // the CG loop's grid barrier
     }
 }
 
@@ -1291,6 +1290,7 @@ __global__ void __launch_bounds__(kFinThreads) k_moments_finalize(Params p, int 
             ts[0] = lambda;
             ts[1] = invW;
         }
+        if (s == 0) *p.bar = 0u;   // the CG loop's grid barrier
         st.rhs2 = a2[0];
         st.rr = a2[1];
         st.sp = a2[2];

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kTileThreads) k_level_rhs(Params p)
         x = ws.v64(s, 0)[i];
     }
     const double cp = st.sumz_l;
+    if (s == 0 && tile == 0 && t == 0) *p.bar = 0u;   // the CG loop's grid barrier
     if (t < 32) {
         double v[2];
         tile_shares(ws.v64(s, 7), p.nblk, v);

@@ -1,0 +1,175 @@
+// Checks of the solve's kernels below the C ABI, linked against the library's own objects:
+//   barrier   the CG loop's grid barrier gives up after its limit when a CTA does not arrive
+//             (and the launch ends), a partial count left in its word does not reach the next
+//             loop, and a loop after a recorded timeout ends at once.
+// Prints one line per check and exits 1 when one fails.
+#include "fbsde_api.cu"
+
+#include <cstdio>
+#include <string>
+
+namespace check {
+
+using fbsde::Layout;
+using fbsde::Params;
+using fbsde::SolveState;
+using LR = fbsde::Launch<float>;
+
+int failures = 0;
+void report(const char *what, bool ok)
+{
+    std::printf("%s: %s\n", what, ok ? "ok" : "FAILED");
+    if (!ok) ++failures;
+}
+#define CUDA_OK(x)                                                                \
+    do {                                                                          \
+        const cudaError_t e_ = (x);                                               \
+        if (e_ != cudaSuccess) {                                                  \
+            std::printf("%s: %s\n", #x, cudaGetErrorString(e_));                  \
+            std::exit(2);                                                         \
+        }                                                                         \
+    } while (0)
+
+// CTAs 1 .. arrive - 1 and CTA 0 meet at the barrier, the others return at once.
+__global__ void k_meet(unsigned int *word, int arrive, unsigned long long limit_ns, int *out,
+                       unsigned long long *ns)
+{
+    __shared__ int flag;
+    if ((int)blockIdx.x >= arrive) return;
+    const unsigned long long t0 = fbsde::dev::globaltimer_ns();
+    const bool ok = fbsde::dev::grid_barrier(word, &flag, limit_ns);
+    if (threadIdx.x == 0) {
+        out[blockIdx.x] = ok ? 1 : 0;
+        ns[blockIdx.x] = fbsde::dev::globaltimer_ns() - t0;
+    }
+}
+
+// A driftless FP32 solve up to the first CG loop, on a workspace of its own.
+struct FirstLoop {
+    Layout L;
+    Params p, ps;
+    char *ws = nullptr;
+    double *x0 = nullptr, *u0 = nullptr;
+    explicit FirstLoop(int d, int M)
+    {
+        fbsde_problem P{};
+        P.kind = FBSDE_AC_MANUFACTURED;
+        P.d = d;
+        P.N = 3;
+        P.M = M;
+        P.sigma = 1.0;
+        P.T = 0.5;
+        P.ridge_rel = 1e-3;
+        P.cg_tol = 1e-7;
+        P.precision = FBSDE_FP32;
+        if (fbsde::make_layout(&P, 1, L) != FBSDE_OK) std::exit(2);
+        CUDA_OK(cudaMalloc(&ws, L.total));
+        CUDA_OK(cudaMemset(ws, 0, L.total));
+        CUDA_OK(cudaMalloc(&x0, d * sizeof(double)));
+        CUDA_OK(cudaMemset(x0, 0, d * sizeof(double)));
+        CUDA_OK(cudaMalloc(&u0, sizeof(double)));
+        p = fbsde::make_params(&P, L, ws, 5, 0, u0, nullptr, nullptr);
+        p.level = P.N;
+        p.newton_level = -1;
+        ps = p;
+        ps.G = L.Gs;
+        CUDA_OK(LR::setup(p, x0, nullptr, 0));
+        CUDA_OK(LR::step(ps, L, 0));
+        CUDA_OK(LR::level_moments(ps, L, 0, 0));
+    }
+    ~FirstLoop()
+    {
+        cudaFree(ws);
+        cudaFree(x0);
+        cudaFree(u0);
+    }
+    Params loop() const
+    {
+        Params q = p;
+        q.level = p.N - 1;
+        return fbsde::product_params(q, L);
+    }
+    std::vector<double> solution() const
+    {
+        std::vector<double> x(L.ld);
+        CUDA_OK(cudaMemcpy(x.data(), p.vec64, L.ld * sizeof(double), cudaMemcpyDeviceToHost));
+        return x;
+    }
+    SolveState state() const
+    {
+        SolveState st;
+        CUDA_OK(cudaMemcpy(&st, p.st, sizeof st, cudaMemcpyDeviceToHost));
+        return st;
+    }
+};
+
+void check_barrier()
+{
+    unsigned int *word;
+    int *out;
+    unsigned long long *ns;
+    CUDA_OK(cudaMalloc(&word, 4));
+    CUDA_OK(cudaMalloc(&out, 4 * sizeof(int)));
+    CUDA_OK(cudaMalloc(&ns, 4 * sizeof(unsigned long long)));
+    for (int arrive : {4, 3}) {
+        CUDA_OK(cudaMemset(word, 0, 4));
+        CUDA_OK(cudaMemset(out, 0, 4 * sizeof(int)));
+        CUDA_OK(cudaMemset(ns, 0, 4 * sizeof(unsigned long long)));
+        unsigned long long limit = 20'000'000ull;
+        void *args[] = {&word, &arrive, &limit, &out, &ns};
+        CUDA_OK(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_meet), dim3(4), dim3(64),
+                                            args, 0, 0));
+        CUDA_OK(cudaDeviceSynchronize());
+        int h[4];
+        unsigned long long t[4];
+        CUDA_OK(cudaMemcpy(h, out, sizeof h, cudaMemcpyDeviceToHost));
+        CUDA_OK(cudaMemcpy(t, ns, sizeof t, cudaMemcpyDeviceToHost));
+        bool ok = true;
+        for (int b = 0; b < arrive; ++b)
+            ok = ok && (arrive == 4 ? h[b] == 1 : h[b] == 0 && t[b] >= limit && t[b] < 10 * limit);
+        report(arrive == 4 ? "barrier of all CTAs" : "barrier with a CTA missing", ok);
+    }
+    CUDA_OK(cudaFree(word));
+    CUDA_OK(cudaFree(out));
+    CUDA_OK(cudaFree(ns));
+
+    std::vector<double> ref;
+    for (unsigned int left : {0u, 1u, 0x80000007u}) {   // the word as a given-up wait leaves it
+        FirstLoop f(300, 900);
+        CUDA_OK(cudaMemcpy(f.p.bar, &left, 4, cudaMemcpyHostToDevice));
+        CUDA_OK(LR::level_rhs(f.ps, f.L, 0));
+        unsigned int word_now = 1;
+        CUDA_OK(cudaMemcpy(&word_now, f.p.bar, 4, cudaMemcpyDeviceToHost));
+        const bool reset = word_now == 0;
+        report("barrier word reset before the loop", reset);
+        if (!reset) return;   // the loop must not run on it
+        CUDA_OK(LR::cg_loop(f.loop(), f.L, 0));
+        CUDA_OK(cudaDeviceSynchronize());
+        const std::vector<double> x = f.solution();
+        const SolveState st = f.state();
+        if (ref.empty()) ref = x;
+        report("loop after a partial count", st.status == 0 && st.done == 1 && st.iters > 1 && x == ref);
+    }
+    {
+        FirstLoop f(300, 900);
+        CUDA_OK(LR::level_rhs(f.ps, f.L, 0));
+        SolveState st = f.state();
+        st.status = FBSDE_ERR_TIMEOUT;
+        CUDA_OK(cudaMemcpy(f.p.st, &st, sizeof st, cudaMemcpyHostToDevice));
+        CUDA_OK(LR::cg_loop(f.loop(), f.L, 0));
+        CUDA_OK(cudaDeviceSynchronize());
+        const SolveState now = f.state();
+        report("loop after a recorded timeout",
+               now.status == FBSDE_ERR_TIMEOUT && now.iters == 0 && now.done == 0);
+    }
+}
+
+}  // namespace check
+
+int main(int argc, char **argv)
+{
+    const std::string what = argc > 1 ? argv[1] : "";
+    if (what == "barrier") check::check_barrier();
+    else return 2;
+    return check::failures ? 1 : 0;
+}
