@@ -642,6 +642,7 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
     const MvTeam m(tw, nteams, nch);
     int phase = 0;
     MvRing rg{0, 0, S, R};   // consumers' position
+    double rr_spec = sc[0].gam;   // of the pass before where phase A runs ahead
     for (int pass = 0;; ++pass) {
         // ---------------- is any query still iterating?
         if (pass == 0 || !spec) {
@@ -690,8 +691,8 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
                     if (c < nch) pc[v] = p.cg_op ? ld_chunk(op + c * E) : ldcg_chunk(pv + c * E);
                     else zero(pc[v]);
                 }
-                RedAcc<Real> dacc;
-                dacc.init();
+                DeltaAcc<Real> dacc;
+                dacc.init(spec ? rr_spec : sc[s].gam);
                 if (resident) rg.slot = rg.par = 0;   // every pass reads the same copy
                 mv_chunk<Real, VPT, (VPT >= 8 && !HOLD), (VPT <= 4 || !HOLD)>(r0, r1, resident ? wsm : ws.w(s) + r0, pv, pc, acc, dacc,
                                            m, ring, full, empty, rg, !resident, slots, phase,
@@ -709,6 +710,7 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
             break;
         }
         // ---------------- phase B
+        rr_spec = sc[0].gam;
         for (int q = NT / 32 - 1 - warp; warp > 0 && q < p.Q; q += NT / 32 - 1) {
             // a tile of query q is this CTA's: the first w >= q nblk with w = blockIdx.x mod
             // gridDim.x lies below (q + 1) nblk

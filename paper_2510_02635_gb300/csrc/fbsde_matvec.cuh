@@ -152,6 +152,41 @@ __device__ __forceinline__ void chunk_axpy(Chunk<float> &y, float a, const Chunk
     y.v[3] = h.y;
 }
 
+// Sum of w t^2 over a team's rows, in the team's first thread.  FP32 rows: compensated, with
+// the rounding errors of both products, of t scaled by a power of two near 1 / |r|: t^2 itself
+// leaves the FP32 range where t does not (sigma = 1e-5: t ~ 1e-20 after a few passes), and
+// 64-bit operations in the row loop cost it 4 to 30%.  FP64 rows: one multiply-add a row.
+template <typename Real> struct DeltaAcc;
+template <> struct DeltaAcc<float> {
+    RedAcc<float> a;
+    float scale;   // 2^-e
+    __device__ __forceinline__ void init(double rr)   // rr: r . r, now or a pass before
+    {
+        a.init();
+        int e = 0;
+        if (rr > 0.0 && isfinite(rr)) e = (((__double2hiint(rr) >> 20) & 0x7FF) - 1023) / 2;
+        e = max(-126, min(126, e));
+        scale = __uint_as_float((uint32_t)(127 - e) << 23);
+    }
+    __device__ __forceinline__ void add(float w, float t)
+    {
+        const float ts = __fmul_rn(t, scale), ws = __fmul_rn(w, ts), h = __fmul_rn(ws, ts);
+        a.add(h);
+        a.c += fmaf(fmaf(w, ts, -ws), ts, fmaf(ws, ts, -h));
+    }
+    __device__ __forceinline__ double value() const
+    {
+        const int e = 127 - (int)(__float_as_uint(scale) >> 23);
+        return a.value() * __hiloint2double((1023 + 2 * e) << 20, 0);   // 4^e
+    }
+};
+template <> struct DeltaAcc<double> {
+    double d;
+    __device__ __forceinline__ void init(double) { d = 0.0; }
+    __device__ __forceinline__ void add(double w, double t) { d += w * t * t; }
+    __device__ __forceinline__ double value() const { return d; }
+};
+
 // NR rows at a time (1 or 2): t = row . r, acc += w t row in row order; the team's first
 // thread adds w t^2 to dacc.  rel0, rel1: "empty" barriers of the stages whose last rows
 // these are (or null); with the rows held in registers they are released before the
@@ -164,7 +199,7 @@ __device__ __forceinline__ void chunk_axpy(Chunk<float> &y, float a, const Chunk
 template <typename Real, int VPT, bool kReread, int NR>
 __device__ __forceinline__ void mv_rows(const Real *const (&row)[NR], const Real (&w)[NR],
                                         const Real *opmem, const Chunk<Real> (&pc)[VPT],
-                                        Chunk<Real> (&acc)[VPT], RedAcc<Real> &dacc, const MvTeam &m,
+                                        Chunk<Real> (&acc)[VPT], DeltaAcc<Real> &dacc, const MvTeam &m,
                                         Real *slots, int &phase, uint64_t *rel0, uint64_t *rel1)
 {
     constexpr int E = Chunk<Real>::E;
@@ -251,7 +286,7 @@ __device__ __forceinline__ void mv_rows(const Real *const (&row)[NR], const Real
 #pragma unroll
     for (int n = 0; n < NR; ++n) {
         const Real coef = w[n] * t[n];
-        if (m.tl == 0) dacc.add(coef * t[n]);   // compensated in FP32: no FP64 in the row loop
+        if (m.tl == 0) dacc.add(w[n], t[n]);
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             if (kReread) dl[n][0] = ld_chunk(row[n] + min(m.tl + m.tthreads * v, m.nch - 1) * E);
@@ -290,7 +325,7 @@ struct MvRing {
 template <typename Real, int VPT, bool kReread, bool kPair>
 __device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real *wv,
                                          const Real *opmem, const Chunk<Real> (&pc)[VPT],
-                                         Chunk<Real> (&acc)[VPT], RedAcc<Real> &dacc, const MvTeam &m,
+                                         Chunk<Real> (&acc)[VPT], DeltaAcc<Real> &dacc, const MvTeam &m,
                                          const Real *ring, uint64_t *full, uint64_t *empty,
                                          MvRing &rg, bool release, Real *slots, int &phase,
                                          bool &timed_out)
@@ -377,7 +412,7 @@ __device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real 
 // r^T A r into dpart.  Called by every consumer thread.
 template <typename Real, int VPT>
 __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const MvTeam &m,
-                                          const Chunk<Real> (&acc)[VPT], const RedAcc<Real> &dacc, Real *red,
+                                          const Chunk<Real> (&acc)[VPT], const DeltaAcc<Real> &dacc, Real *red,
                                           double *dsl)
 {
     constexpr int E = Chunk<Real>::E;
@@ -489,8 +524,8 @@ __global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512)
             else zero(pc[v]);
         }
         int phase = 0;
-        RedAcc<Real> dacc;
-        dacc.init();
+        DeltaAcc<Real> dacc;
+        dacc.init(p.st[s].rr);
         MvRing rg{0, 0, S, R};
         mv_chunk<Real, VPT, (MODE != kMvHold), (VPT <= 8 && (VPT <= 4 || MODE != kMvHold))>(r0, r1, ws.w(s) + r0, pv, pc, acc, dacc, m, ring, full,
                                                empty, rg, true, slots, phase, timed_out);

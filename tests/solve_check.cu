@@ -2,6 +2,8 @@
 //   barrier   the CG loop's grid barrier gives up after its limit when a CTA does not arrive
 //             (and the launch ends), a partial count left in its word does not reach the next
 //             loop, and a loop after a recorded timeout ends at once.
+//   delta     the product's shares of r^T A r, sum_j w_j (D_j . r)^2, against the same sum in
+//             long double, on rows and operands whose dot products are exact in FP32.
 // Prints one line per check and exits 1 when one fails.
 #include "fbsde_api.cu"
 
@@ -164,12 +166,60 @@ void check_barrier()
     }
 }
 
+// Rows and r of small integers (r scaled by a power of two): every dot product t is exact in
+// FP32, in any order.  The sums are compensated FP32 sums with the products' rounding errors:
+// n rows a team leave (n 2^-24)^2 of them (Neumaier's bound), and the products' second-order
+// errors 4 2^-48.
+void check_delta(int d, int M)
+{
+    for (float scale : {1.0f, 0x1p-70f, 0x1p50f}) {
+        FirstLoop f(d, M);
+        const Layout &L = f.L;
+        std::vector<float> rows((size_t)M * L.ld), r(L.ld), w(M);
+        uint32_t seed = 12345;
+        auto next = [&] { return (seed = seed * 1664525u + 1013904223u) >> 8; };
+        for (int i = 0; i < L.ld; ++i) r[i] = i < d ? scale * (float)((int)(next() % 7) - 3) : 0.0f;
+        long double want = 0.0L;
+        for (int j = 0; j < M; ++j) {
+            w[j] = (float)next() * 0x1p-24f;
+            long double t = 0.0L;
+            for (int i = 0; i < L.ld; ++i) {
+                const float x = i < d ? (float)((int)(next() % 7) - 3) : 0.0f;
+                rows[(size_t)j * L.ld + i] = x;
+                t += (long double)x * r[i];
+            }
+            want += (long double)w[j] * t * t;
+        }
+        CUDA_OK(cudaMemcpy(f.p.delta, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice));
+        CUDA_OK(cudaMemcpy(f.p.vecR, r.data(), r.size() * 4, cudaMemcpyHostToDevice));
+        CUDA_OK(cudaMemcpy(f.p.w, w.data(), w.size() * 4, cudaMemcpyHostToDevice));
+        SolveState st = f.state();
+        st.rr = 0.0;
+        for (float v : r) st.rr += (double)v * v;
+        CUDA_OK(cudaMemcpy(f.p.st, &st, sizeof st, cudaMemcpyHostToDevice));
+        const Params q = f.loop();
+        CUDA_OK(LR::matvec(q, L, 0));
+        CUDA_OK(cudaDeviceSynchronize());
+        std::vector<double> share((size_t)L.Gc * fbsde::kDpart);
+        CUDA_OK(cudaMemcpy(share.data(), q.dpart, share.size() * 8, cudaMemcpyDeviceToHost));
+        double got = 0.0;
+        for (int g = 0; g < L.Gc; ++g) got += share[(size_t)g * fbsde::kDpart];
+        const double err = std::fabs((double)(((long double)got - want) / want));
+        std::printf("d %d M %d scale %.1e: error %.1e (%d chunks, %d teams)\n", d, M, scale, err, L.Gc,
+                    L.teams);
+        const double n = (M + L.Gc * L.teams - 1) / (L.Gc * L.teams) + 1.0;
+        report("delta", err <= (n * n + 4.0) * 0x1p-48);
+    }
+}
+
 }  // namespace check
 
 int main(int argc, char **argv)
 {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "barrier") check::check_barrier();
+    else if (what == "delta")   // several teams; chunks of more than 32 rows a team; one team a row
+        for (auto [d, M] : {std::pair{301, 900}, {33, 90001}, {5003, 4001}}) check::check_delta(d, M);
     else return 2;
     return check::failures ? 1 : 0;
 }
