@@ -34,17 +34,25 @@ bool choose_team(int nch, bool resident, int &tw, int &vpt)
     return 32 * tw <= 512;
 }
 
+// Bytes of one team's sums of earlier runs (fbsde_matvec.cuh) in a product of G chunks.
+size_t mv_runs_bytes(const fbsde_problem *P, int G, int teams, size_t row_bytes)
+{
+    return P->precision == FBSDE_FP32 && teams == 1 && (P->M + G - 1) / G > dev::kMvRun ? row_bytes : 0;
+}
+
 // Ring of a product launch of G chunks per query: S stages of R rows, about 32 KB a stage and
 // 200 KB of shared memory in all.  A CTA never needs a ring larger than its own rows: small
 // instances keep their ring, and so their shared memory, small (two stages of at most half
 // their rows), which lets the CTAs of concurrent instances share an SM.
+// runs: bytes wanted beside the ring (fewer stages where both do not fit).
 void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, size_t real_sz,
-                  int &rows, int &stages, size_t &smem)
+                  size_t runs, int &rows, int &stages, size_t &smem)
 {
     const size_t stage_target = 32 * 1024, ring_target = 200 * 1024;
     long long R = std::max<long long>(1, (long long)(stage_target / row_bytes));
     R = std::max<long long>(teams, R / teams * teams);
     long long S = std::min<long long>(8, std::max<long long>(2, ring_target / (R * row_bytes)));
+    if (runs) S = std::max<long long>(2, std::min<long long>(S, (220 * 1024 - runs) / (R * row_bytes)));
     const long long rows_cta = (P->M + G - 1) / G;
     if (S * R > rows_cta) {
         const long long half = ((rows_cta + 1) / 2 + teams - 1) / teams * teams;
@@ -53,7 +61,8 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
     }
     rows = (int)R;
     stages = (int)S;
-    smem = (size_t)S * R * row_bytes + 2 * S * sizeof(uint64_t) + (size_t)teams * 2 * 32 * real_sz;
+    smem = (size_t)S * R * row_bytes + 2 * S * sizeof(uint64_t) +
+           (size_t)teams * 2 * 32 * real_sz + runs;
 }
 
 // Geometry of the CG (fbsde_cg.cuh): teams, chunks, tiles and the loop's shared memory; all
@@ -62,6 +71,13 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 //   - Chunks: without a given ctas, as many waves of 152 chunks (one per SM) over the
 //     queries as fill the SMs best, no chunk below one row per team (four rows for one
 //     team: a chunk's partial vector is written and read like a row).
+//   - Runs: a thread adds its rows' FP32 products uncompensated, the partial vectors are added
+//     compensated.  FP32 chunks of several teams have at most kTeamRun rows a team, in more waves
+//     if need be (and not in shared memory for the whole loop): slopes against the FP64 path,
+//     M = 16384, one query: d = 2468, 36 rows a team, 2.6e-6 as with 18; d = 4005, 54 rows
+//     5.1e-6, 27 rows 4.6e-6.  One team adds longer chunks in runs of kMvRun rows instead: more
+//     partial vectors of its wide rows cost more (d = 10^4, M = 16384, one query, three levels:
+//     18.3 ms with 608 of them, 15.5 ms with 152 in runs).
 //   - A chunk that fits the loop's shared memory stays there for the whole loop; then up
 //     to 14 warps share its rows, which hides the latency of
 //     a row's dot product.  Rows that stream through the ring instead get as many teams as
@@ -70,6 +86,7 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 //     the partial vectors of a tile are added by one CTA, so more tiles shorten phase B.
 constexpr size_t kCgSmem = 225 * 1024;   // dynamic shared memory of the loop
 constexpr long long kCgSms = 152;
+constexpr long long kTeamRun = 40;
 
 bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
 {
@@ -84,11 +101,18 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
         1, std::min<long long>(warps / L.team_warps, 96 * 1024 / (long long)row));
     const size_t tile_sm = L.precision == FBSDE_FP32 ? sizeof(dev::CgTileSm<float>)
                                                      : sizeof(dev::CgTileSm<double>);
+    auto runs = [&](int teams) { return mv_runs_bytes(P, L.Gc, teams, row); };
     auto fixed = [&](int teams, long long ring_rows, int stages) {   // all but the ring
         L.cg_op = teams > 1 ? 1 : 0;
-        L.cg_both = (int)align_up(std::max(tile_sm, teams > 1 ? teams * row : 0), 16);
+        L.cg_both = (int)align_up(std::max(tile_sm, teams > 1 ? teams * row : runs(teams)), 16);
         return (size_t)L.cg_op * row + L.cg_both + Q * sizeof(dev::CgScal) + 16 * (size_t)stages +
                ((size_t)teams * 64 + ring_rows) * L.real_sz + 128;
+    };
+    const int gcap = kPartVecs * std::max(L.G, L.Gs);   // the partial vectors' buffer
+    // chunks of a query at least, for runs of kTeamRun rows of a team
+    auto least = [&](int teams) {
+        const long long rows = kTeamRun * teams;
+        return P->precision == FBSDE_FP32 && P->ctas == 0 && teams > 1 ? (P->M + rows - 1) / rows : 1LL;
     };
     auto chunks = [&](int teams, bool one_wave) {
         const long long gmax =
@@ -105,15 +129,18 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
             }
             if (g == gmax) break;
         }
+        if (!one_wave && G < least(teams)) {
+            const long long W = (least(teams) * Q + kCgSms - 1) / kCgSms;
+            G = (int)std::min<long long>({gmax, gcap, std::max(least(teams), kCgSms * W / Q)});
+        }
         return G;
     };
-    const int gcap = kPartVecs * std::max(L.G, L.Gs);   // the partial vectors' buffer
     int wmax = warps;
     L.cg_res = 0;
     L.teams = tmax;
     L.Gc = std::min(gcap, chunks(tmax, true));
     long long rows = (P->M + L.Gc - 1) / L.Gc;
-    if ((long long)Q * L.Gc <= kCgSms && L.team_warps <= warps && L.vpt <= 8 &&
+    if ((long long)Q * L.Gc <= kCgSms && L.Gc >= least(tmax) && L.team_warps <= warps && L.vpt <= 8 &&
         rows * row + fixed(tmax, rows, 2) <= kCgSmem) {
         L.cg_res = 1;
         L.cg_stages = rows > tmax ? 2 : 1;
@@ -149,7 +176,7 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
         while (L.c3_vpt < 8 && 32 * L.c3_vpt < nch) L.c3_vpt *= 2;
         L.c3_tw = (nch + 32 * L.c3_vpt - 1) / (32 * L.c3_vpt);
         L.c3_teams = std::max(1, 256 / (32 * L.c3_tw));
-        product_ring(P, row, L.G, L.c3_teams, 4, L.c3_rows, L.c3_stages, L.c3_smem);
+        product_ring(P, row, L.G, L.c3_teams, 4, 0, L.c3_rows, L.c3_stages, L.c3_smem);
         if (L.c3_tw > 16 || L.c3_smem > 227 * 1024) return false;
     }
     L.mv_mode = L.team_warps > 10 ? dev::kMvWide : (L.teams > 1 ? dev::kMvHold : dev::kMvPair);
@@ -372,7 +399,8 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
         place();
     }
     if (!cg_geometry(P, Q, L)) return FBSDE_ERR_ARG;
-    product_ring(P, (size_t)L.ld * L.real_sz, L.Gc, L.teams, L.real_sz, L.mv_rows, L.mv_stages,
+    product_ring(P, lds * L.real_sz, L.Gc, L.teams, L.real_sz,
+                 mv_runs_bytes(P, L.Gc, L.teams, lds * L.real_sz), L.mv_rows, L.mv_stages,
                  L.mv_smem);
     if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
     // reverse sweep: tape of the primal plus three adjoint vectors per query

@@ -694,10 +694,10 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
                 DeltaAcc<Real> dacc;
                 dacc.init(spec ? rr_spec : sc[s].gam);
                 if (resident) rg.slot = rg.par = 0;   // every pass reads the same copy
-                mv_chunk<Real, VPT, (VPT >= 8 && !HOLD), (VPT <= 4 || !HOLD)>(r0, r1, resident ? wsm : ws.w(s) + r0, pv, pc, acc, dacc,
-                                           m, ring, full, empty, rg, !resident, slots, phase,
-                                           timed_out);
-                mv_finish<Real, VPT>(p, s, g, m, acc, dacc, red, dsl);
+                const bool flushed = mv_chunk<Real, VPT, (VPT >= 8 && !HOLD), (VPT <= 4 || !HOLD)>(
+                    r0, r1, red, resident ? wsm : ws.w(s) + r0, pv, pc, acc, dacc, m, ring,
+                    full, empty, rg, !resident, slots, phase, timed_out);
+                mv_finish<Real, VPT>(p, s, g, m, acc, flushed, dacc, red, dsl);
                 // op and red are written again only past the barriers of the next chunk
             }
         }

@@ -306,6 +306,11 @@ __device__ __forceinline__ void mv_rows(const Real *const (&row)[NR], const Real
 //   kMvWide  as kMvPair with teams of 11 to 16 warps.
 enum MvMode { kMvHold = 0, kMvPair = 1, kMvWide = 2 };
 
+// Rows of a chunk that a thread adds up in FP32 before the sum goes on elsewhere: an FP32 run of n
+// rows loses about sqrt(n) roundings.  d = 5003, M = 16000, one query: slopes 7.2e-6 from the
+// FP64 path with runs of 105 rows, 5.8e-6 with 32.
+constexpr int kMvRun = 32;
+
 // Position of a consumer in the ring of row stages.
 struct MvRing {
     int slot, par, S, R;
@@ -318,12 +323,30 @@ struct MvRing {
     }
 };
 
+// The thread's chunks of `sum` (shared memory) added to its accumulators.
+template <typename Real, int VPT>
+__device__ __forceinline__ void mv_add_runs(const Real *sum, const MvTeam &m, Chunk<Real> (&acc)[VPT])
+{
+    constexpr int E = Chunk<Real>::E;
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        const int c = m.tl + m.tthreads * v;
+        if (c < m.nch) {
+            const Chunk<Real> o = ld_chunk(sum + c * E);
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[v].v[e] += o.v[e];
+        }
+    }
+}
+
 // The consumers' part of one chunk, rows [r0, r1): its stages of R rows (a multiple of the
 // teams) from the ring, released after use unless they stay (release = false).  wv: the
 // weights from row r0 on.  kPair: two rows of a team at a time (of two stages where a stage
-// holds one row per team).
+// holds one row per team).  One team that reads its FP32 rows again: every kMvRun rows the
+// accumulators go into `sum` ([ld] in shared memory, each thread its own chunks); returns whether
+// they did.
 template <typename Real, int VPT, bool kReread, bool kPair>
-__device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real *wv,
+__device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, const Real *wv,
                                          const Real *opmem, const Chunk<Real> (&pc)[VPT],
                                          Chunk<Real> (&acc)[VPT], DeltaAcc<Real> &dacc, const MvTeam &m,
                                          const Real *ring, uint64_t *full, uint64_t *empty,
@@ -347,7 +370,22 @@ __device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real 
     // the weights of the team's next two rows, requested one step ahead of their use
     auto weight = [&](int j) { return j < nrows ? wv[j] : Real(0); };
     Real n0 = weight(m.team), n1 = weight(m.team + nt);
+    // (rows of one team that are read again come one a stage, or a few of them stay resident)
+    constexpr bool kRuns = sizeof(Real) == 4 && kReread;
+    bool flushed = false;
+    int run = 0;
     for (int base = 0; base < nrows;) {
+        if (kRuns && run >= kMvRun) {
+            if (flushed) mv_add_runs<Real, VPT>(sum, m, acc);
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                const int c = m.tl + m.tthreads * v;
+                if (c < m.nch) st_chunk(sum + c * Chunk<Real>::E, acc[v]);
+                zero(acc[v]);
+            }
+            flushed = true;
+            run = 0;
+        }
         const int a = rg.slot, rows = min(rg.R, nrows - base);
         const Real *buf = ring + (size_t)a * rg.R * ld;
         uint64_t *ea = release ? &empty[a] : nullptr;
@@ -381,6 +419,7 @@ __device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real 
                 }
             }
             base += two ? 2 * rg.R : rg.R;
+            run += 2;
             continue;
         }
         int rr = m.team;
@@ -405,14 +444,16 @@ __device__ __forceinline__ void mv_chunk(long long r0, long long r1, const Real 
         }
         base += rg.R;
     }
+    return flushed;
 }
 
 // The chunk's results: the teams' accumulators added in team order (through red,
 // [nteams][ld], free for the consumers' use) into partial g, and the teams' shares of
-// r^T A r into dpart.  Called by every consumer thread.
+// r^T A r into dpart.  flushed: one team's earlier runs are in red.  Called by every consumer
+// thread.
 template <typename Real, int VPT>
 __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const MvTeam &m,
-                                          const Chunk<Real> (&acc)[VPT], const DeltaAcc<Real> &dacc, Real *red,
+                                          Chunk<Real> (&acc)[VPT], bool flushed, const DeltaAcc<Real> &dacc, Real *red,
                                           double *dsl)
 {
     constexpr int E = Chunk<Real>::E;
@@ -420,6 +461,7 @@ __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const M
     Real *dst = ws.part(s, g, 0);
     double *dp = p.dpart + ((size_t)s * p.G + g) * kDpart;
     if (m.nteams == 1) {
+        if (flushed) mv_add_runs<Real, VPT>(red, m, acc);
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             const int c = m.tl + m.tthreads * v;
@@ -482,6 +524,7 @@ __global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512)
     uint64_t *full = reinterpret_cast<uint64_t *>(ring + (size_t)S * R * row_elems);
     uint64_t *empty = full + S;
     Real *slots = reinterpret_cast<Real *>(empty + S);                   // [nteams][2][32]
+    Real *runs = slots + (size_t)nteams * 64;                            // [ld] of one team
     long long r0, r1;
     row_range(p.M, p.G, g, r0, r1);
     const long long nst = (r1 - r0 + R - 1) / R;
@@ -527,10 +570,12 @@ __global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512)
         DeltaAcc<Real> dacc;
         dacc.init(p.st[s].rr);
         MvRing rg{0, 0, S, R};
-        mv_chunk<Real, VPT, (MODE != kMvHold), (VPT <= 8 && (VPT <= 4 || MODE != kMvHold))>(r0, r1, ws.w(s) + r0, pv, pc, acc, dacc, m, ring, full,
-                                               empty, rg, true, slots, phase, timed_out);
+        const bool flushed =
+            mv_chunk<Real, VPT, (MODE != kMvHold), (VPT <= 8 && (VPT <= 4 || MODE != kMvHold))>(
+                r0, r1, runs, ws.w(s) + r0, pv, pc, acc, dacc, m, ring, full, empty, rg,
+                true, slots, phase, timed_out);
         if (nteams > 1) bar_named(15, m.tthreads * nteams);   // past the last ring read
-        mv_finish<Real, VPT>(p, s, g, m, acc, dacc, ring, dsl);
+        mv_finish<Real, VPT>(p, s, g, m, acc, flushed, dacc, flushed ? runs : ring, dsl);
     }
     if (timed_out) atomicCAS(&p.st[s].status, 0, (int)FBSDE_ERR_TIMEOUT);
 }

@@ -4,6 +4,8 @@
 //             loop, and a loop after a recorded timeout ends at once.
 //   delta     the product's shares of r^T A r, sum_j w_j (D_j . r)^2, against the same sum in
 //             long double, on rows and operands whose dot products are exact in FP32.
+//   runs      the product's FP32 sums over long chunks, on rows of which one is 2^25 times the
+//             others: only the rest of its run is lost beside it.
 // Prints one line per check and exits 1 when one fails.
 #include "fbsde_api.cu"
 
@@ -212,6 +214,49 @@ void check_delta(int d, int M)
     }
 }
 
+// Every row has D_0 = 1 and r = e_0, so t = w = 1 and coordinate 1 of a chunk's partial vector is
+// the sum of the rows' D_1: 1 in the chunk's first row and 2^-25 in the others.  In FP32 the 1
+// swallows what is added to it one by one: the other kMvRun - 1 rows of its run (one unit of
+// 2^-25 each); after that every addition to it rounds by two units at most, one for each further
+// run of the team and for each other team.
+void check_runs(int d, int M)
+{
+    FirstLoop f(d, M);
+    const Layout &L = f.L;
+    std::vector<float> rows((size_t)M * L.ld, 0.0f), r(L.ld, 0.0f), w(M, 1.0f);
+    r[0] = 1.0f;
+    std::vector<int> count(L.Gc);
+    for (int g = 0; g < L.Gc; ++g) {
+        const long long r0 = (long long)M * g / L.Gc, r1 = (long long)M * (g + 1) / L.Gc;
+        count[g] = (int)(r1 - r0);
+        for (long long j = r0; j < r1; ++j) {
+            rows[(size_t)j * L.ld] = 1.0f;
+            rows[(size_t)j * L.ld + 1] = j == r0 ? 1.0f : 0x1p-25f;
+        }
+    }
+    CUDA_OK(cudaMemcpy(f.p.delta, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice));
+    CUDA_OK(cudaMemcpy(f.p.vecR, r.data(), r.size() * 4, cudaMemcpyHostToDevice));
+    CUDA_OK(cudaMemcpy(f.p.w, w.data(), w.size() * 4, cudaMemcpyHostToDevice));
+    const Params q = f.loop();
+    CUDA_OK(LR::matvec(q, L, 0));
+    CUDA_OK(cudaDeviceSynchronize());
+    std::vector<float> part((size_t)L.Gc * L.ld);
+    CUDA_OK(cudaMemcpy(part.data(), q.part, part.size() * 4, cudaMemcpyDeviceToHost));
+    double worst = 0.0;
+    bool ok = true;
+    const int run = fbsde::dev::kMvRun;
+    for (int g = 0; g < L.Gc; ++g) {
+        const double exact = 1.0 + (count[g] - 1) * 0x1p-25;
+        const double lost = std::fabs(part[(size_t)g * L.ld + 1] - exact) * 0x1p25;   // units
+        const int team = (count[g] + L.teams - 1) / L.teams;
+        ok = ok && lost <= run - 1 + 2 * ((team - 1) / run) + 2 * (L.teams - 1);
+        worst = std::max(worst, lost);
+    }
+    std::printf("d %d M %d: %d chunks of %d rows, %d teams, resident %d: %.0f units lost\n", d, M, L.Gc,
+                count[0], L.teams, L.cg_res, worst);
+    report("runs", ok && (L.teams > 1 || count[0] > 4 * run));
+}
+
 }  // namespace check
 
 int main(int argc, char **argv)
@@ -220,6 +265,8 @@ int main(int argc, char **argv)
     if (what == "barrier") check::check_barrier();
     else if (what == "delta")   // several teams; chunks of more than 32 rows a team; one team a row
         for (auto [d, M] : {std::pair{301, 900}, {33, 90001}, {5003, 4001}}) check::check_delta(d, M);
+    else if (what == "runs")   // one team a row; several, streaming and in shared memory
+        for (auto [d, M] : {std::pair{5003, 20011}, {33, 456007}, {4, 900001}}) check::check_runs(d, M);
     else return 2;
     return check::failures ? 1 : 0;
 }

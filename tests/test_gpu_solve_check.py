@@ -28,3 +28,7 @@ def test_grid_barrier_gives_up_and_leaves_no_count(program):
 
 def test_shares_of_delta_keep_twice_fp32(program):
     _run(program, "delta", 9)
+
+
+def test_long_chunks_are_added_in_runs(program):
+    _run(program, "runs", 3)
