@@ -1302,16 +1302,17 @@ struct TcColumnsEpi {
         s.v[0] = t;
         return s;
     }
-    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<1> &s) const
+    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<1> (&s)[4]) const
     {
-        part[((size_t)tile * M + m) * 3] = (double)s.v[0];
+        part[((size_t)tile * M + m) * 3] = (double)(((s[0].v[0] + s[1].v[0]) + s[2].v[0]) + s[3].v[0]);
     }
 };
 
 // Epilogue of the distances' product P A^T on the tensor cores: the weights and the column
 // sums of w, w Y and w rho over each 128-row tile, straight from the accumulator
 // (k_anc_columns in mode 0, fused: the product is neither written nor read back; 25 us of a
-// level at d = 100, M = 2048).  Tiles off the band are not visited: the caller keeps W zero
+// level at d = 100, M = 2048).  FP32 sums of 32 rows, widened before they are added on (the
+// column pass widens its sums of 64).  Tiles off the band are not visited: the caller keeps W zero
 // there, and the sums' readers skip them.
 struct TcWeightsEpi {
     const double *pn, *an, *Y;
@@ -1345,12 +1346,12 @@ struct TcWeightsEpi {
         W[(size_t)j * M + m] = w;
         return s;
     }
-    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<3> &s) const
+    __device__ __forceinline__ void colsum(int tile, int m, const dev::TcSums<3> (&s)[4]) const
     {
         double *o = part + ((size_t)tile * M + m) * 3;
-        o[0] = (double)s.v[0];
-        o[1] = (double)s.v[1];
-        o[2] = (double)s.v[2];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            o[i] = ((double)s[0].v[i] + (double)s[1].v[i]) + ((double)s[2].v[i] + (double)s[3].v[i]);
     }
 };
 

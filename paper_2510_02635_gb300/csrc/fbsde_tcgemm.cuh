@@ -236,7 +236,7 @@ struct TcStore {
         C[((size_t)z * Mr + row) * ldc + col] = v;
         return {};
     }
-    __device__ __forceinline__ void colsum(int, int, const TcSums<0> &) const {}
+    __device__ __forceinline__ void colsum(int, int, const TcSums<0> (&)[4]) const {}
 };
 
 // Sum_k A(r, k) B(c, k) over k in [z kc, min(K, (z + 1) kc)) for split z = blockIdx.z
@@ -246,8 +246,8 @@ struct TcStore {
 // Epi::prefetch(r0, c, column state, pre) for the 32 rows r0.. a warp hands out next
 // (issued before the accumulator is read, so its loads overlap that),
 // Epi::put(z, r, c, value, column state, pre, r - r0), whose Epi::kSums return values are
-// summed over the rows of the block's 128-row tile (rows in order, 32-row quarters in order)
-// and passed to Epi::colsum(row tile, c, sums).  stop (or null): a word that, when not 0, ends
+// summed over the rows of each 32-row quarter of the block's 128-row tile (rows in order); the
+// quarters' sums go to Epi::colsum(row tile, c, sums), which adds them as it needs.  stop (or null): a word that, when not 0, ends
 // the launch at once (a pass behind the last one of a loop).
 // Grid (ceil(Nc / 128), ceil(Mr / 128), splits), kTcThreads threads, kTcSmemBytes of
 // dynamic shared memory.  A wait that times out sets *status = FBSDE_ERR_TIMEOUT (if 0).
@@ -383,12 +383,11 @@ __global__ void __launch_bounds__(kTcThreads, 3)
         __syncthreads();
         const int t = threadIdx.x;
         if (t < kTcBN && c0 + t < Nc) {
-            TcSums<Epi::kSums> sum;
+            TcSums<Epi::kSums> sum[4];
 #pragma unroll
-            for (int i = 0; i < Epi::kSums; ++i) {
-                const float *c = csm + 4 * i * kTcBN + t;
-                sum.v[i] = ((c[0] + c[kTcBN]) + c[2 * kTcBN]) + c[3 * kTcBN];
-            }
+            for (int i = 0; i < Epi::kSums; ++i)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sum[u].v[i] = csm[(4 * i + u) * kTcBN + t];
             epi.colsum(blockIdx.y, c0 + t, sum);
         }
     }

@@ -1,4 +1,4 @@
-"""Compiles tests/solve_check.cu against the library's sources and objects."""
+"""Compiles the check programs of tests/ against the library's sources and objects."""
 import os
 import shutil
 import subprocess
@@ -14,15 +14,23 @@ def nvcc():
     return cand if os.path.exists(cand) else shutil.which("nvcc")
 
 
+def _compile(source, directory, objs=()) -> str:
+    exe = os.path.join(str(directory), source[:-3])
+    cmd = [nvcc(), "-std=c++17", "-O2", "-gencode", "arch=compute_103a,code=sm_103a",
+           "-I", os.path.join(ROOT, "include"), "-I", gbuild.CSRC, os.path.join(HERE, source),
+           *objs, "-o", exe]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    return exe
+
+
+def compile_anchored_check(directory) -> str:
+    return _compile("anchored_check.cu", directory)
+
+
 def compile_solve_check(directory) -> str:
     gbuild.build()
     objs = [os.path.join(gbuild.BUILD, f) for f in ("fbsde_kernels_f32.o", "fbsde_kernels_f64.o")]
     if not all(os.path.exists(o) for o in objs):   # a library that came without its objects
         gbuild.build(force=True)
-    exe = os.path.join(str(directory), "solve_check")
-    cmd = [nvcc(), "-std=c++17", "-O2", "-gencode", "arch=compute_103a,code=sm_103a",
-           "-I", os.path.join(ROOT, "include"), "-I", gbuild.CSRC,
-           os.path.join(HERE, "solve_check.cu"), *objs, "-o", exe]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr[-3000:]
-    return exe
+    return _compile("solve_check.cu", directory, objs)
