@@ -2,24 +2,29 @@
 
 The tunable is `ctas`: how many CTAs one streaming pass over a query's particle cloud
 uses (rows per CTA = M / ctas).  Wide tilings fill the GPU for one large instance;
-narrow ones leave SMs to the other instances of a concurrent batch.  The tuner times a
-short probe solve (same d, M and kind, N_probe levels) through a one-instance plan for
-each candidate and keeps the narrowest tiling within `slack` of the fastest, per
-(log2 d, M) bucket; results are cached as JSON.  All timing is on the GPU with CUDA
-events; nothing here computes any part of the method.
+narrow ones leave SMs to the other instances of a concurrent batch; 0 is the library's own
+tiling.  The tuner times a short probe solve (same d, M and kind, N_probe levels) for each
+candidate and keeps the narrowest tiling within `slack` of the fastest, per (log2 d, M) bucket.
+The probe is a plan of two copies on two branches: the CG of a plan with several branches runs
+as separate launches, that of a plan with one branch as one cooperative launch over the GPU
+with other tilings to its liking.  Results are cached as JSON with a hash of the library that
+was timed; another library's are timed again.  All timing is on the GPU with CUDA events;
+nothing here computes any part of the method.
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import math
 import os
 
 import numpy as np
 
-from . import fbsde
+from . import build, fbsde
 from . import workloads as W
 
-CANDIDATES = (76, 152, 304, 608, 1216)
+CANDIDATES = (0, 76, 152, 304, 608, 1216)
+DEFAULT_CTAS = 608   # of the streaming passes with ctas = 0 (fbsde.h): 0 counts as this wide
 DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build",
                              "autotune.json")
 
@@ -78,14 +83,30 @@ def _time_plan(plan, torch, repeats: int) -> float:
     return ev0.elapsed_time(ev1) / repeats
 
 
+def _library_hash() -> str:
+    with open(build.LIB, "rb") as fh:
+        return hashlib.sha256(fh.read()).hexdigest()[:16]
+
+
+def _cached(cache_path: str | None, library: str) -> dict:
+    if not cache_path or not os.path.exists(cache_path):
+        return {}
+    try:
+        with open(cache_path) as fh:
+            data = json.load(fh)
+    except ValueError:
+        return {}
+    if not isinstance(data, dict) or data.get("library") != library:
+        return {}
+    return data["table"]
+
+
 def tune(instances: list[W.Workload], cache_path: str | None = DEFAULT_CACHE,
          n_probe: int = 2, repeats: int = 2, slack: float = 1.10) -> dict:
     """ctas per bucket for the given instances (cached)."""
     import torch
-    table = {}
-    if cache_path and os.path.exists(cache_path):
-        with open(cache_path) as fh:
-            table = json.load(fh)
+    library = _library_hash()
+    table = _cached(cache_path, library)
     todo = {}
     for w in instances:
         todo.setdefault(bucket(w), w)
@@ -99,17 +120,19 @@ def tune(instances: list[W.Workload], cache_path: str | None = DEFAULT_CACHE,
             if c > max(1, w.M // 8) * 2:   # more CTAs than row blocks: same as the cap
                 continue
             p = problem_of(w, ctas=c, N=min(n_probe, w.N))
-            plan = fbsde.Plan([{"problem": p, "Q": 1, "x0": x0, "seed": w.seed}])
+            plan = fbsde.Plan([{"problem": p, "Q": 1, "x0": x0, "seed": w.seed,
+                                "solve_index0": i} for i in range(2)], branches=2)
             times[c] = _time_plan(plan, torch, repeats)
             plan.close()
         best = min(times.values())
-        chosen = min(c for c, t in times.items() if t <= slack * best)
+        chosen = min((c for c, t in times.items() if t <= slack * best),
+                     key=lambda c: (c or DEFAULT_CTAS, c))
         table[key] = {"ctas": chosen, "probe_ms": {str(c): t for c, t in times.items()}}
         changed = True
     if changed and cache_path:
         os.makedirs(os.path.dirname(cache_path), exist_ok=True)
         with open(cache_path, "w") as fh:
-            json.dump(table, fh, indent=1, sort_keys=True)
+            json.dump({"library": library, "table": table}, fh, indent=1, sort_keys=True)
     return table
 
 
