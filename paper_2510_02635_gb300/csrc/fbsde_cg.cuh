@@ -23,7 +23,10 @@
 namespace fbsde {
 namespace dev {
 
-constexpr int kCgThreads = 512;   // threads of k_cg_tile
+// Threads of k_cg_tile and k_level_moments: a warp for the scalars beside those that read the
+// partials; FP32 blocks of 56 registers, three an SM (two of 512 threads and 64 registers before:
+// 65 queries, d = 700: 18.9 -> 14.1 us a launch).
+constexpr int kCgThreads = 384;
 constexpr int kCgWarps = 10;      // warps 1..10 read a tile's partials (warp 0 waits at the
                                   // grid barrier, and its first loads after that are slow)
 constexpr int kCgQueries = 64;    // most queries of k_cg_loop (every CTA keeps their scalars)
@@ -416,7 +419,7 @@ __device__ __forceinline__ bool cg_arrive(const Params &p, int s, const CgScal &
 // finish sets the while-loop condition: 1 while some query has not converged and fewer than
 // cg_max_iter passes ran (with one query, its last tile does so without a second arrival).
 template <typename Real>
-__global__ void __launch_bounds__(kCgThreads) k_cg_tile(Params p, cudaGraphConditionalHandle h,
+__global__ void __launch_bounds__(kCgThreads, sizeof(Real) == 4 ? 3 : 2) k_cg_tile(Params p, cudaGraphConditionalHandle h,
                                                         int use_h)
 {
     __shared__ CgTileSm<Real> sm;
