@@ -34,10 +34,12 @@ bool choose_team(int nch, bool resident, int &tw, int &vpt)
     return 32 * tw <= 512;
 }
 
-// Bytes of one team's sums of earlier runs (fbsde_matvec.cuh) in a product of G chunks.
-size_t mv_runs_bytes(const fbsde_problem *P, int G, int teams, size_t row_bytes)
+// Bytes of the teams' sums of earlier runs (fbsde_matvec.cuh) in a product of G chunks.
+size_t mv_runs_bytes(const fbsde_problem *P, int G, int teams, int vpt, size_t row_bytes)
 {
-    return P->precision == FBSDE_FP32 && teams == 1 && (P->M + G - 1) / G > dev::kMvRun ? row_bytes : 0;
+    return P->precision == FBSDE_FP32 && (teams == 1 || vpt == 1) &&
+                   (P->M + G - 1) / G > (long long)dev::kMvRun * teams
+               ? teams * row_bytes : 0;
 }
 
 // Ring of a product launch of G chunks per query: S stages of R rows, about 32 KB a stage and
@@ -72,12 +74,13 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 //     queries as fill the SMs best, no chunk below one row per team (four rows for one
 //     team: a chunk's partial vector is written and read like a row).
 //   - Runs: a thread adds its rows' FP32 products uncompensated, the partial vectors are added
-//     compensated.  FP32 chunks of several teams have at most kTeamRun rows a team, in more waves
-//     if need be (and not in shared memory for the whole loop): slopes against the FP64 path,
-//     M = 16384, one query: d = 2468, 36 rows a team, 2.6e-6 as with 18; d = 4005, 54 rows
-//     5.1e-6, 27 rows 4.6e-6.  One team adds longer chunks in runs of kMvRun rows instead: more
-//     partial vectors of its wide rows cost more (d = 10^4, M = 16384, one query, three levels:
-//     18.3 ms with 608 of them, 15.5 ms with 152 in runs).
+//     compensated.  One team per row, and rows of one chunk per thread, add long chunks in runs of
+//     kMvRun rows.  (More partial vectors instead cost more: d = 10^4, M = 16384, one query, three
+//     levels: 18.3 ms with 608 of them, 15.5 ms with 152 in runs.)  Several teams of wider rows,
+//     whose registers are short, have at most kTeamRun rows a team instead, in more waves if need
+//     be, in clouds of fewer than kRunRatio d rows, whose regressions amplify the rounding: slopes
+//     against the FP64 path, M = 16384, one query: d = 2468, 36 rows a team, 2.6e-6 as with 18;
+//     d = 4005, 54 rows 5.1e-6, 27 rows 4.6e-6; d = 2000, M = 65536: 8.2e-6 with 108 and with 36.
 //   - A chunk that fits the loop's shared memory stays there for the whole loop; then up
 //     to 14 warps share its rows, which hides the latency of
 //     a row's dot product.  Rows that stream through the ring instead get as many teams as
@@ -86,7 +89,7 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 //     the partial vectors of a tile are added by one CTA, so more tiles shorten phase B.
 constexpr size_t kCgSmem = 225 * 1024;   // dynamic shared memory of the loop
 constexpr long long kCgSms = 152;
-constexpr long long kTeamRun = 40;
+constexpr long long kTeamRun = 40, kRunRatio = 16;
 
 bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
 {
@@ -101,7 +104,7 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
         1, std::min<long long>(warps / L.team_warps, 96 * 1024 / (long long)row));
     const size_t tile_sm = L.precision == FBSDE_FP32 ? sizeof(dev::CgTileSm<float>)
                                                      : sizeof(dev::CgTileSm<double>);
-    auto runs = [&](int teams) { return mv_runs_bytes(P, L.Gc, teams, row); };
+    auto runs = [&](int teams) { return mv_runs_bytes(P, L.Gc, teams, L.vpt, row); };
     auto fixed = [&](int teams, long long ring_rows, int stages) {   // all but the ring
         L.cg_op = teams > 1 ? 1 : 0;
         L.cg_both = (int)align_up(std::max(tile_sm, teams > 1 ? teams * row : runs(teams)), 16);
@@ -112,7 +115,9 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
     // chunks of a query at least, for runs of kTeamRun rows of a team
     auto least = [&](int teams) {
         const long long rows = kTeamRun * teams;
-        return P->precision == FBSDE_FP32 && P->ctas == 0 && teams > 1 ? (P->M + rows - 1) / rows : 1LL;
+        return P->precision == FBSDE_FP32 && P->ctas == 0 && teams > 1 && L.vpt > 1 &&
+                       P->M < kRunRatio * P->d
+                   ? (P->M + rows - 1) / rows : 1LL;
     };
     auto chunks = [&](int teams, bool one_wave) {
         const long long gmax =
@@ -140,7 +145,7 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
     L.teams = tmax;
     L.Gc = std::min(gcap, chunks(tmax, true));
     long long rows = (P->M + L.Gc - 1) / L.Gc;
-    if ((long long)Q * L.Gc <= kCgSms && L.Gc >= least(tmax) && L.team_warps <= warps && L.vpt <= 8 &&
+    if ((long long)Q * L.Gc <= kCgSms && L.team_warps <= warps && L.vpt <= 8 &&
         rows * row + fixed(tmax, rows, 2) <= kCgSmem) {
         L.cg_res = 1;
         L.cg_stages = rows > tmax ? 2 : 1;
@@ -400,7 +405,7 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
     }
     if (!cg_geometry(P, Q, L)) return FBSDE_ERR_ARG;
     product_ring(P, lds * L.real_sz, L.Gc, L.teams, L.real_sz,
-                 mv_runs_bytes(P, L.Gc, L.teams, lds * L.real_sz), L.mv_rows, L.mv_stages,
+                 mv_runs_bytes(P, L.Gc, L.teams, L.vpt, lds * L.real_sz), L.mv_rows, L.mv_stages,
                  L.mv_smem);
     if (L.mv_smem > 227 * 1024) return FBSDE_ERR_ARG;
     // reverse sweep: tape of the primal plus three adjoint vectors per query

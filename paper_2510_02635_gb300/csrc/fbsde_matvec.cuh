@@ -342,9 +342,9 @@ __device__ __forceinline__ void mv_add_runs(const Real *sum, const MvTeam &m, Ch
 // The consumers' part of one chunk, rows [r0, r1): its stages of R rows (a multiple of the
 // teams) from the ring, released after use unless they stay (release = false).  wv: the
 // weights from row r0 on.  kPair: two rows of a team at a time (of two stages where a stage
-// holds one row per team).  One team that reads its FP32 rows again: every kMvRun rows the
-// accumulators go into `sum` ([ld] in shared memory, each thread its own chunks); returns whether
-// they did.
+// holds one row per team).  FP32 rows of one team that reads them again, or of one chunk per thread:
+// every kMvRun rows of a team its accumulators go into its row of `sum` ([nteams][ld] in shared
+// memory, each thread its own chunks); returns whether they did.
 template <typename Real, int VPT, bool kReread, bool kPair>
 __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, const Real *wv,
                                          const Real *opmem, const Chunk<Real> (&pc)[VPT],
@@ -370,22 +370,27 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
     // the weights of the team's next two rows, requested one step ahead of their use
     auto weight = [&](int j) { return j < nrows ? wv[j] : Real(0); };
     Real n0 = weight(m.team), n1 = weight(m.team + nt);
-    // (rows of one team that are read again come one a stage, or a few of them stay resident)
-    constexpr bool kRuns = sizeof(Real) == 4 && kReread;
+    // Runs end at the team's row 32, 64, ..: a pair never straddles two, so that they do not
+    // depend on the stages.  (Rows of one team that are read again come one a stage, where run
+    // stays even, or a few of them stay resident.)
+    constexpr bool kRuns = sizeof(Real) == 4 && kReread, kRunsIn = sizeof(Real) == 4 && VPT == 1;
+    Real *const mine = sum + (size_t)m.team * ld;
     bool flushed = false;
     int run = 0;
-    for (int base = 0; base < nrows;) {
-        if (kRuns && run >= kMvRun) {
-            if (flushed) mv_add_runs<Real, VPT>(sum, m, acc);
+    auto next_run = [&]() {   // before a row of the team
+        if (run < kMvRun) return;
+        if (flushed) mv_add_runs<Real, VPT>(mine, m, acc);
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                const int c = m.tl + m.tthreads * v;
-                if (c < m.nch) st_chunk(sum + c * Chunk<Real>::E, acc[v]);
-                zero(acc[v]);
-            }
-            flushed = true;
-            run = 0;
+        for (int v = 0; v < VPT; ++v) {
+            const int c = m.tl + m.tthreads * v;
+            if (c < m.nch) st_chunk(mine + c * Chunk<Real>::E, acc[v]);
+            zero(acc[v]);
         }
+        flushed = true;
+        run = 0;
+    };
+    for (int base = 0; base < nrows;) {
+        if (kRuns || (kRunsIn && across && base + m.team < nrows)) next_run();
         const int a = rg.slot, rows = min(rg.R, nrows - base);
         const Real *buf = ring + (size_t)a * rg.R * ld;
         uint64_t *ea = release ? &empty[a] : nullptr;
@@ -426,22 +431,31 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
         mbar_wait_or_flag(&full[a], (uint32_t)rg.par, timed_out);
         rg.next();
         if (rr >= rows) none(ea, nullptr);
-        if constexpr (kPair) {
-            for (; rr + nt < rows; rr += 2 * nt) {
-                const Real w[2] = {n0, n1};
-                const Real *const row[2] = {buf + (size_t)rr * ld, buf + (size_t)(rr + nt) * ld};
-                n0 = weight(base + rr + 2 * nt);
-                n1 = weight(base + rr + 3 * nt);
-                mv_rows<Real, VPT, kReread, 2>(row, w, opmem, pc, acc, dacc, m, slots, phase,
-                                               rr + 2 * nt < rows ? nullptr : ea, nullptr);
+        do {
+            int end = rows;   // rows of this stage and run
+            if (kRunsIn) {
+                if (rr < rows) next_run();
+                end = min(rows, rr + (kMvRun - run) * nt);
             }
-        }
-        for (; rr < rows; rr += nt) {
-            const Real w = n0;
-            n0 = n1;
-            n1 = weight(base + rr + 2 * nt);
-            one(buf + (size_t)rr * ld, w, rr + nt < rows ? nullptr : ea);
-        }
+            if constexpr (kPair) {
+                for (; rr + nt < end; rr += 2 * nt) {
+                    const Real w[2] = {n0, n1};
+                    const Real *const row[2] = {buf + (size_t)rr * ld, buf + (size_t)(rr + nt) * ld};
+                    n0 = weight(base + rr + 2 * nt);
+                    n1 = weight(base + rr + 3 * nt);
+                    mv_rows<Real, VPT, kReread, 2>(row, w, opmem, pc, acc, dacc, m, slots, phase,
+                                                   rr + 2 * nt < rows ? nullptr : ea, nullptr);
+                    if (kRunsIn) run += 2;
+                }
+            }
+            for (; rr < end; rr += nt) {
+                const Real w = n0;
+                n0 = n1;
+                n1 = weight(base + rr + 2 * nt);
+                one(buf + (size_t)rr * ld, w, rr + nt < rows ? nullptr : ea);
+                if (kRunsIn) ++run;
+            }
+        } while (kRunsIn && rr < rows);
         base += rg.R;
     }
     return flushed;
@@ -449,7 +463,7 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
 
 // The chunk's results: the teams' accumulators added in team order (through red,
 // [nteams][ld], free for the consumers' use) into partial g, and the teams' shares of
-// r^T A r into dpart.  flushed: one team's earlier runs are in red.  Called by every consumer
+// r^T A r into dpart.  flushed: the team's earlier runs are in red.  Called by every consumer
 // thread.
 template <typename Real, int VPT>
 __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const MvTeam &m,
@@ -460,8 +474,8 @@ __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const M
     const WS<Real> ws(p);
     Real *dst = ws.part(s, g, 0);
     double *dp = p.dpart + ((size_t)s * p.G + g) * kDpart;
+    if (flushed) mv_add_runs<Real, VPT>(red + (size_t)m.team * m.nch * E, m, acc);
     if (m.nteams == 1) {
-        if (flushed) mv_add_runs<Real, VPT>(red, m, acc);
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             const int c = m.tl + m.tthreads * v;
@@ -524,7 +538,7 @@ __global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512)
     uint64_t *full = reinterpret_cast<uint64_t *>(ring + (size_t)S * R * row_elems);
     uint64_t *empty = full + S;
     Real *slots = reinterpret_cast<Real *>(empty + S);                   // [nteams][2][32]
-    Real *runs = slots + (size_t)nteams * 64;                            // [ld] of one team
+    Real *runs = slots + (size_t)nteams * 64;                            // [nteams][ld]
     long long r0, r1;
     row_range(p.M, p.G, g, r0, r1);
     const long long nst = (r1 - r0 + R - 1) / R;
@@ -575,7 +589,10 @@ __global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512)
                 r0, r1, runs, ws.w(s) + r0, pv, pc, acc, dacc, m, ring, full, empty, rg,
                 true, slots, phase, timed_out);
         if (nteams > 1) bar_named(15, m.tthreads * nteams);   // past the last ring read
-        mv_finish<Real, VPT>(p, s, g, m, acc, flushed, dacc, flushed ? runs : ring, dsl);
+        // the same for every team, and as the host counts (mv_runs_bytes)
+        const bool own = sizeof(Real) == 4 && (nteams == 1 || VPT == 1) &&
+                         r1 - r0 > (long long)kMvRun * nteams;
+        mv_finish<Real, VPT>(p, s, g, m, acc, flushed, dacc, own ? runs : ring, dsl);
     }
     if (timed_out) atomicCAS(&p.st[s].status, 0, (int)FBSDE_ERR_TIMEOUT);
 }
