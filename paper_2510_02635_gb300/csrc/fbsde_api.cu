@@ -72,7 +72,9 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 // device.
 //   - Chunks: without a given ctas, as many waves of 152 chunks (one per SM) over the
 //     queries as fill the SMs best, no chunk below one row per team (four rows for one
-//     team: a chunk's partial vector is written and read like a row).
+//     team: a chunk's partial vector is written and read like a row); further waves as long as
+//     their chunks have kWaveRows rows (33 queries, d = 1932, 151 rows: 2.10 ms with 23 chunks a
+//     query, 1.81 ms with 9).
 //   - Runs: a thread adds its rows' FP32 products uncompensated, the partial vectors are added
 //     compensated.  One team per row, and rows of one chunk per thread, add long chunks in runs of
 //     kMvRun rows.  (More partial vectors instead cost more: d = 10^4, M = 16384, one query, three
@@ -89,6 +91,7 @@ void product_ring(const fbsde_problem *P, size_t row_bytes, int G, int teams, si
 //     the partial vectors of a tile are added by one CTA, so more tiles shorten phase B.
 constexpr size_t kCgSmem = 225 * 1024;   // dynamic shared memory of the loop
 constexpr long long kCgSms = 152;
+constexpr long long kWaveRows = 16;
 constexpr long long kTeamRun = 40, kRunRatio = 16;
 
 bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
@@ -127,6 +130,7 @@ bool cg_geometry(const fbsde_problem *P, int Q, Layout &L)
         int G = 1;
         for (int W = 1; W <= (one_wave ? 1 : 8); ++W) {
             const long long g = std::min(gmax, std::max<long long>(1, kCgSms * W / Q));
+            if (W > 1 && g * kWaveRows > P->M) break;
             const double waves = (double)(g * Q) / kCgSms, eff = waves / std::ceil(waves);
             if (eff > best + 0.015) {
                 best = eff;

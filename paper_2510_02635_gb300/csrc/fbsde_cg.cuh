@@ -23,7 +23,7 @@
 namespace fbsde {
 namespace dev {
 
-// Threads of k_cg_tile and k_level_moments: a warp for the scalars beside those that read the
+// Threads of k_cg_tile (at most) and k_level_moments: a warp for the scalars beside those that read the
 // partials; FP32 blocks of 56 registers, three an SM (two of 512 threads and 64 registers before:
 // 65 queries, d = 700: 18.9 -> 14.1 us a launch).
 constexpr int kCgThreads = 384;
@@ -431,11 +431,11 @@ __global__ void __launch_bounds__(kCgThreads, sizeof(Real) == 4 ? 3 : 2) k_cg_ti
     if (st.done) {
         answer = blockIdx.x == 0 && threadIdx.x == 0;   // one block answers for a finished query
     } else {
-        if (threadIdx.x >= kCgThreads - 32) {   // a warp that reads no partials
+        if (threadIdx.x >= blockDim.x - 32) {   // a warp that reads no partials
             CgScal c = cg_load(st);
             cg_prepare(c);
             cg_step_scalar<Real>(p, s, c, c.a, c.ok);
-            if (threadIdx.x == kCgThreads - 32) sc = c;
+            if (threadIdx.x == blockDim.x - 32) sc = c;
         }
         __syncthreads();
         cg_tile<Real, kCgThreads>(p, s, blockIdx.x, sc, sm);

@@ -254,7 +254,11 @@ template <typename Real>
 cudaError_t Launch<Real>::cg_tile(const Params &p, const Layout &L, cudaGraphConditionalHandle h,
                                   int use_h, cudaStream_t s)
 {
-    dev::k_cg_tile<Real><<<dim3(L.cg_nblk, L.Q), dev::kCgThreads, 0, s>>>(p, h, use_h);
+    // warp 0, the warps that read partials or own coordinates, the scalars' warp: few partials
+    // (small clouds) take small blocks, more of them an SM
+    const int per = 32 / L.cg_lpr, parts = std::min(dev::kCgWarps, (L.Gc + per - 1) / per);
+    const int warps = 2 + std::max(parts, (4 * L.cg_lpr + 31) / 32);
+    dev::k_cg_tile<Real><<<dim3(L.cg_nblk, L.Q), 32 * warps, 0, s>>>(p, h, use_h);
     return cudaGetLastError();
 }
 

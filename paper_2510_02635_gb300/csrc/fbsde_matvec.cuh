@@ -519,7 +519,8 @@ __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const M
 // which lets the producer refill it.
 // MODE (MvMode): how a team walks its rows; set with the geometry.
 template <typename Real, int VPT, int MODE>
-__global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512), 1)
+__global__ void __launch_bounds__(MODE == kMvWide ? 544 : (VPT >= 8 ? 352 : 512),
+                                  VPT == 1 && sizeof(Real) == 4 ? 2 : 1)
     k_matvec(Params p)
 {
     constexpr int E = Chunk<Real>::E;
