@@ -296,7 +296,7 @@ int make_layout(const fbsde_problem *P, int32_t Q, Layout &L)
         L.st_R = 1;
         L.st_T = 480;
         double best_rate = 0.0;
-        for (int T : {16, 32, 64, 96, 128, 160, 192, 288}) {
+        for (int T : {16, 32, 64, 96, 128, 160, 192}) {
             const int vm = (nch + T - 1) / T;
             long long R = std::min<long long>({kStepMaxConsumers / T, kStepElems / L.ld, 30});
             if (T < 32) R &= ~1LL;   // whole warps

@@ -2,10 +2,11 @@
 // vectors, vector updates.  Included after fbsde_cg.cuh.  It keeps the wide tiling of the
 // product (608 CTAs over the queries, one partial each) and forms delta = w . r from the
 // reduced product, so a pass has two exchanges instead of one.  It serves the shapes whose
-// passes are long enough not to feel that: several queries of rows above 16 KB that stream
-// from HBM, rows too wide for the loop's block, and the forward SDE, whose slopes are a small
-// remainder of a large mean shift (their rounding shows in the fifth digit, so its sums keep
-// this order).  Measured: d = 10^4, M = 16384, 16 queries, 338.0 ms for five levels here and
+// passes are long enough not to feel that, wherever the loop is not taken and a row has one team
+// (rows above 16 KB): several queries whose rows stream from HBM, rows too wide for the loop's
+// block (d > 10240), more than 64 queries (also of small clouds); and the forward SDE, whose
+// slopes are a small remainder of a large mean shift (their rounding shows in the fifth digit, so
+// its sums keep this order).  Measured: d = 10^4, M = 16384, 16 queries, 338.0 ms for five levels here and
 // 338.2 ms in two launches (product 1390 and 1375 us).
 #pragma once
 #include "fbsde_cg.cuh"
@@ -69,19 +70,13 @@ __global__ void __launch_bounds__(WIDE ? 544 : (VPT >= 8 ? 352 : 288), 1) k_prod
         const int team = ct / tthreads, tl = ct - team * tthreads, wt = tl >> 5;
         const Real *pv = ws.vR(s, 0);
         const Real *wv = ws.w(s);
-        // the operand r: in registers, except with 16 chunks per thread (the widest FP64
-        // rows), where it is read through L1 for every row (it is the same for all rows)
-        constexpr bool kOpL1 = VPT > 8;
-        constexpr int kOpRegs = kOpL1 ? 1 : VPT;
-        Chunk<Real> acc[VPT], pc[kOpRegs];
+        Chunk<Real> acc[VPT], pc[VPT];   // pc: the operand r
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             zero(acc[v]);
-            if (!kOpL1) {
-                const int c = tl + tthreads * v;
-                if (c < nch) pc[v] = ldg_chunk(pv + c * E);
-                else zero(pc[v]);
-            }
+            const int c = tl + tthreads * v;
+            if (c < nch) pc[v] = ldg_chunk(pv + c * E);
+            else zero(pc[v]);
         }
         int phase = 0;
         for (long long i = 0; i < nst; ++i) {
@@ -97,9 +92,9 @@ __global__ void __launch_bounds__(WIDE ? 544 : (VPT >= 8 ? 352 : 288), 1) k_prod
                 const Real wrow = wv[row0 + rr];
                 // narrow teams keep their chunks of the row in registers between the dot
                 // product and the weighted sum (one shared-memory read of the row instead
-                // of two); the 16-warp teams of the widest rows, and the 16 chunks per
-                // thread of the widest FP64 rows, have no registers to spare
-                constexpr bool kReread = WIDE || VPT > 8;
+                // of two); the 11- to 16-warp teams of the widest rows have no registers to
+                // spare
+                constexpr bool kReread = WIDE;
                 constexpr int kHeld = kReread ? 1 : VPT;
                 Chunk<Real> dl[kHeld];
                 Real t = Real(0);
@@ -107,16 +102,10 @@ __global__ void __launch_bounds__(WIDE ? 544 : (VPT >= 8 ? 352 : 288), 1) k_prod
                 for (int v = 0; v < VPT; ++v) {
                     const int c = tl + tthreads * v;
                     Chunk<Real> &x = dl[kReread ? 0 : v];
-                    Chunk<Real> &o = pc[kOpL1 ? 0 : v];
-                    if (c < nch) {
-                        x = ld_chunk(row + c * E);
-                        if (kOpL1) o = ldg_chunk(pv + c * E);
-                    } else {
-                        zero(x);
-                        if (kOpL1) zero(o);
-                    }
+                    if (c < nch) x = ld_chunk(row + c * E);
+                    else zero(x);
 #pragma unroll
-                    for (int e = 0; e < E; ++e) t += x.v[e] * o.v[e];
+                    for (int e = 0; e < E; ++e) t += x.v[e] * pc[v].v[e];
                 }
 #pragma unroll
                 for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);

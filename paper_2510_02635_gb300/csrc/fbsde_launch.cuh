@@ -230,7 +230,9 @@ cudaError_t Launch<Real>::matvec(const Params &p, const Layout &L, cudaStream_t 
         switch (L.mv_mode) {
         case dev::kMvHold: return launch_matvec<Real, 8, dev::kMvHold>(p, L, s);
         case dev::kMvPair: return launch_matvec<Real, 8, dev::kMvPair>(p, L, s);
-        case dev::kMvWide: return launch_matvec<Real, 8, dev::kMvWide>(p, L, s);
+        case dev::kMvWide:   // FP64; FP32 rows of such teams take the pass in three launches
+            if constexpr (sizeof(Real) == 8) return launch_matvec<Real, 8, dev::kMvWide>(p, L, s);
+            break;
         }
         return cudaErrorInvalidValue;
     case 16:   // FP64 rows of 8193 to 10240 values: teams of 9 or 10 warps
