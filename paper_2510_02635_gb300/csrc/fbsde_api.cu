@@ -1239,10 +1239,11 @@ size_t fbsde_plan_workspace_bytes(int32_t n, const fbsde_instance *inst)
     return plan_layout(n, inst, v, total) == FBSDE_OK ? total : 0;
 }
 
-// Scheduling model of a CG pass for the plan's branches: the launches of a pass (product,
-// reduction, update) cost about 25 us however small the instance, and its rows stream at
-// about 6.5 TB/s.
-constexpr double kPassLatency = 25e-6;
+// Scheduling model of a CG pass for the plan's branches: the launches of a pass (product and
+// tiles in the conditional node) cost about 20 us however small the instance (d = 148, M = 512:
+// 18 us a pass with two branches, 20 us with eight, the levels' other kernels included; 25 us
+// with the three launches before), and its rows stream at about 6.5 TB/s.
+constexpr double kPassLatency = 20e-6;
 constexpr double kPassBandwidth = 6.5e12;
 
 int fbsde_plan_create(fbsde_plan **plan, int32_t n, const fbsde_instance *inst, int32_t branches,
