@@ -417,15 +417,14 @@ typedef struct {
    timed launch adds two event records to its stream, so timing only the family of
    interest keeps the profiler's own cost out of the rest of the step.  ERR_ARG for a
    mask with no valid family bit. */
-/* How the eager entry points (fbsde_solve, fbsde_solve_host, fbsde_adjoint) launch the
-   passes of a CG loop (fbsde_solve_noalloc always launches every pass, up to cg_max_iter,
-   one by one on the stream, so that it creates no CUDA graph): while the profiler times the product
-   family, the first FBSDE_PROFILED_EAGER_PASSES passes of every loop are launched one by
-   one (each product launch bracketed by events; kernels of converged queries exit at
-   once) and any further passes run in a cached CUDA graph whose conditional while loop
-   stops when every query has converged.  Otherwise every pass of a loop runs in one
-   cooperative launch, or, for the shapes that it does not serve, in that graph.  On a
-   stream that is being captured these are launched one by one, up to cg_max_iter passes.
+/* How the eager entry points launch the passes of a CG loop: every pass of a loop in one
+   cooperative launch, or, for the shapes that it does not serve and on a stream whose SMs
+   do not hold it, in a cached CUDA graph whose conditional while loop stops when every
+   query has converged; on a stream that is being captured, and in fbsde_solve_noalloc,
+   which creates no CUDA graph, the passes of those shapes are launched one by one, up to
+   cg_max_iter (kernels of converged queries exit at once).  While the profiler times the
+   product family, the first FBSDE_PROFILED_EAGER_PASSES passes of every loop are launched
+   one by one, each product launch bracketed by events, and any further ones as above.
    The results are the same bit for bit in every case. */
 #define FBSDE_PROFILED_EAGER_PASSES 48
 FBSDE_API int fbsde_profile_start(int32_t max_timed_launches);

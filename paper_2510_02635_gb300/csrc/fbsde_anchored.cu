@@ -1203,7 +1203,7 @@ bool lay(const fbsde_problem *P, Lay &L)
     L.P = take(M * ld * L.rs);
     L.A = take(M * ld * L.rs);
     L.YP = take(M * ld * L.rs);
-    L.G1 = take(M * M * L.rs);
+    L.G1 = take(M * M * L.rs);   // (unused by FP32 with M >= 1024, whose epilogues replace it)
     L.W = take(M * M * L.rs);
     L.T = take(M * M * L.rs);
     L.G2 = take((size_t)L.nsplit * M * ld * L.rs);

@@ -1073,8 +1073,8 @@ __global__ void k_philox(const uint32_t *ctr, const uint32_t *key, uint32_t *out
 }  // namespace fbsde
 
 namespace fbsde {
-// fbsde_solve with every CG pass launched on the stream (no CUDA graph is created,
-// instantiated or cached), for the entry point that must allocate nothing.
+// fbsde_solve by launches on the stream alone (no CUDA graph is created, instantiated or
+// cached), for the entry point that must allocate nothing.
 int solve_launches_only(const fbsde_problem *P, int32_t Q, const double *x0, uint64_t seed,
                         uint32_t solve_index0, double *u0, double *grad_u0, void *workspace,
                         size_t workspace_bytes, cudaStream_t stream)

@@ -30,8 +30,8 @@
 
 namespace fbsde {
 
-// fbsde_solve with every CG pass launched on the stream, creating no CUDA graph
-// (fbsde_api.cu); used by the entry point without a workspace argument.
+// fbsde_solve by launches on the stream alone, creating no CUDA graph (fbsde_api.cu); used by
+// the entry point without a workspace argument.
 int solve_launches_only(const fbsde_problem *P, int32_t Q, const double *x0, uint64_t seed,
                         uint32_t solve_index0, double *u0, double *grad_u0, void *workspace,
                         size_t workspace_bytes, cudaStream_t stream);
@@ -78,8 +78,8 @@ struct Layout {
     size_t mv_smem;
     // CG: row chunks per query of the product, lanes per row of partials and tiles of phase
     // B; the loop's ring (rows per stage, stages, rows in all), whether it holds a CTA's rows for the
-    // whole loop, bytes of its operand (0 or 1 row), shared sums and shared memory; cg_ok:
-    // the loop covers this shape
+    // whole loop, rows of its operand (0 or 1), bytes of the sums of both phases and of shared
+    // memory; cg_ok: the loop covers this shape
     int mv_mode, Gc, cg_lpr, cg_nblk, cg_rows, cg_stages, cg_ring, cg_res, cg_op, cg_both, cg_ok;
     size_t cg_smem;
     // the pass in three launches (fbsde_cg3.cuh) instead, with its own team geometry and ring

@@ -13,7 +13,7 @@
 //   rows above about 3400 floats  R = 1, T = 480 (15 consumer warps and one service warp,
 //                    128 registers a thread), a ring of two stages;
 //   narrower rows    R >= 3, R T <= 576 (up to 18 consumer warps and two service warps, 96
-//                    registers), a ring of 3 to 8 stages.
+//                    registers), a ring of 4 to 8 stages.
 //   load (a service warp, one lane)  the rows Delta_{k+1} of a stage are copied into the
 //                    shared-memory ring by one bulk copy (cp.async.bulk, completion on the
 //                    slot's mbarrier) as soon as the consumers are done with the slot;
