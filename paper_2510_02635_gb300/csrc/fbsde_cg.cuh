@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
     __shared__ double dsl[16];
     __shared__ int flag;
     __shared__ CgProducer pr;
-    if (__ldcg(&p.st[0].status) == FBSDE_ERR_TIMEOUT) return;
+    const int before = __ldcg(&p.st[0].status);   // of the solve so far; checked below
     const WS<Real> ws(p);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = p.ld / E, S = p.cg_stages, R = p.cg_rows;
@@ -570,6 +570,7 @@ __global__ void __launch_bounds__(NT, 1) k_cg_loop(Params p)
         for (int j = threadIdx.x; j < (int)(r1 - r0); j += NT) wsm[j] = ws.w(s)[r0 + j];
     }
     __syncthreads();
+    if (before == FBSDE_ERR_TIMEOUT) return;
     bool timed_out = false;
     // producer (thread 0): its state lives in shared memory, out of the consumers' registers
     if (threadIdx.x == 0) {

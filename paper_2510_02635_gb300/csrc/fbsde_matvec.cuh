@@ -160,12 +160,13 @@ template <typename Real> struct DeltaAcc;
 template <> struct DeltaAcc<float> {
     RedAcc<float> a;
     float scale;   // 2^-e
-    __device__ __forceinline__ void init(double rr)   // rr: r . r, now or a pass before
+    // rr: r . r, now or a pass before; only its exponent counts (integer arithmetic:
+    // FP64 comparisons in every warp held the SM's FP64 pipe for 0.3 us a pass at d = 64)
+    __device__ __forceinline__ void init(double rr)
     {
         a.init();
-        int e = 0;
-        if (rr > 0.0 && isfinite(rr)) e = (((__double2hiint(rr) >> 20) & 0x7FF) - 1023) / 2;
-        e = max(-126, min(126, e));
+        const int f = (__double2hiint(rr) >> 20) & 0xFFF;   // sign and exponent
+        const int e = f > 0 && f < 0x7FF ? max(-126, min(126, (f - 1023) / 2)) : 0;
         scale = __uint_as_float((uint32_t)(127 - e) << 23);
     }
     __device__ __forceinline__ void add(float w, float t)
@@ -174,10 +175,13 @@ template <> struct DeltaAcc<float> {
         a.add(h);
         a.c += fmaf(fmaf(w, ts, -ws), ts, fmaf(ws, ts, -h));
     }
-    __device__ __forceinline__ double value() const
+    __device__ __forceinline__ double value() const { return a.value(); }   // scaled by 4^-e
+    // A sum of such values times 4^e, by its exponent (0, infinities and NaN stay)
+    __device__ __forceinline__ double back(double d) const
     {
         const int e = 127 - (int)(__float_as_uint(scale) >> 23);
-        return a.value() * __hiloint2double((1023 + 2 * e) << 20, 0);   // 4^e
+        const int hi = __double2hiint(d), f = (hi >> 20) & 0x7FF;
+        return f == 0 || f == 0x7FF ? d : __hiloint2double(hi + ((2 * e) << 20), __double2loint(d));
     }
 };
 template <> struct DeltaAcc<double> {
@@ -185,6 +189,7 @@ template <> struct DeltaAcc<double> {
     __device__ __forceinline__ void init(double) { d = 0.0; }
     __device__ __forceinline__ void add(double w, double t) { d += w * t * t; }
     __device__ __forceinline__ double value() const { return d; }
+    __device__ __forceinline__ double back(double v) const { return v; }
 };
 
 // NR rows at a time (1 or 2): t = row . r, acc += w t row in row order; the team's first
@@ -481,7 +486,7 @@ __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const M
             const int c = m.tl + m.tthreads * v;
             if (c < m.nch) st_chunk(dst + c * E, acc[v]);
         }
-        if (m.tl == 0) *dp = dacc.value();
+        if (m.tl == 0) *dp = dacc.back(dacc.value());
         return;
     }
     const int nthreads = m.tthreads * m.nteams;
@@ -499,7 +504,7 @@ __device__ __forceinline__ void mv_finish(const Params &p, int s, int g, const M
         double d = m.lane < m.nteams ? dsl[m.lane] : 0.0;
 #pragma unroll
         for (int o = 8; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (m.lane == 0) *dp = d;
+        if (m.lane == 0) *dp = dacc.back(d);
     }
     for (int c = ct; c < m.nch; c += nthreads) {
         Chunk<Real> sum = ld_chunk(red + c * E);
