@@ -56,11 +56,11 @@ def instance_cost(w) -> float:
     """Estimated time of one instance, in seconds: N levels of 2 + sqrt(kappa) passes over
     its rows (the row step and the moments, then CG passes growing like the square root of
     the regression's condition number kappa, estimated from the Marchenko-Pastur edges of
-    the cloud's covariance and the ridge), each pass a fixed launch latency of 25 us plus
+    the cloud's covariance and the ridge), each pass a fixed launch latency of 20 us plus
     its rows at 6.5 TB/s.  The plan's branch scheduler uses the same model."""
     from .autotune import kappa_estimate
     nbytes = float(w.Q) * w.M * w.d * (4.0 if w.precision == "fp32" else 8.0)
-    return w.N * (2.0 + math.sqrt(kappa_estimate(w))) * (25e-6 + nbytes / 6.5e12)
+    return w.N * (2.0 + math.sqrt(kappa_estimate(w))) * (20e-6 + nbytes / 6.5e12)
 
 
 def cost_shard(instances, world: int) -> list[list[int]]:
