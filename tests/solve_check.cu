@@ -169,9 +169,8 @@ void check_barrier()
 }
 
 // Rows and r of small integers (r scaled by a power of two): every dot product t is exact in
-// FP32, in any order.  The sums are compensated FP32 sums with the products' rounding errors:
-// n rows a team leave (n 2^-24)^2 of them (Neumaier's bound), and the products' second-order
-// errors 4 2^-48.
+// FP32, in any order.  Each term w t^2 has two FP32 roundings, 2 2^-24 of it at most; the sums
+// are compensated, n rows a team leave (n 2^-24)^2 of them (Neumaier's bound).
 void check_delta(int d, int M)
 {
     for (float scale : {1.0f, 0x1p-70f, 0x1p50f}) {
@@ -210,7 +209,7 @@ void check_delta(int d, int M)
         std::printf("d %d M %d scale %.1e: error %.1e (%d chunks, %d teams)\n", d, M, scale, err, L.Gc,
                     L.teams);
         const double n = (M + L.Gc * L.teams - 1) / (L.Gc * L.teams) + 1.0;
-        report("delta", err <= (n * n + 4.0) * 0x1p-48);
+        report("delta", err <= 0x1.00001p-23 + n * n * 0x1p-48);
     }
 }
 

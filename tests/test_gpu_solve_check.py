@@ -1,6 +1,6 @@
 """Kernels of the solve below the C ABI (tests/solve_check.cu, compiled here and run): the
 bounded waits of the CG loop's grid barrier and what a wait that gave up leaves behind, and the
-precision and range of the product's shares of r^T A r."""
+range of the product's shares of r^T A r."""
 import subprocess
 
 import pytest
@@ -26,7 +26,7 @@ def test_grid_barrier_gives_up_and_leaves_no_count(program):
     _run(program, "barrier", 9)
 
 
-def test_shares_of_delta_keep_twice_fp32(program):
+def test_shares_of_delta_keep_their_range(program):
     _run(program, "delta", 9)
 
 
