@@ -380,6 +380,7 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
     // depend on the stages.  (Rows of one team that are read again come one a stage, where run
     // stays even, or a few of them stay resident.)
     constexpr bool kRuns = sizeof(Real) == 4 && kReread, kRunsIn = sizeof(Real) == 4 && VPT == 1;
+    const bool more = kRunsIn && nrows > kMvRun * nt;   // a team has more than one run
     Real *const mine = sum + (size_t)m.team * ld;
     bool flushed = false;
     int run = 0;
@@ -396,7 +397,7 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
         run = 0;
     };
     for (int base = 0; base < nrows;) {
-        if (kRuns || (kRunsIn && across && base + m.team < nrows)) next_run();
+        if (kRuns || (more && across && base + m.team < nrows)) next_run();
         const int a = rg.slot, rows = min(rg.R, nrows - base);
         const Real *buf = ring + (size_t)a * rg.R * ld;
         uint64_t *ea = release ? &empty[a] : nullptr;
@@ -439,7 +440,7 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
         if (rr >= rows) none(ea, nullptr);
         do {
             int end = rows;   // rows of this stage and run
-            if (kRunsIn) {
+            if (more) {
                 if (rr < rows) next_run();
                 end = min(rows, rr + (kMvRun - run) * nt);
             }
@@ -461,7 +462,7 @@ __device__ __forceinline__ bool mv_chunk(long long r0, long long r1, Real *sum, 
                 one(buf + (size_t)rr * ld, w, rr + nt < rows ? nullptr : ea);
                 if (kRunsIn) ++run;
             }
-        } while (kRunsIn && rr < rows);
+        } while (more && rr < rows);
         base += rg.R;
     }
     return flushed;
